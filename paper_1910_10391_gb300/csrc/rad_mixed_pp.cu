@@ -467,7 +467,9 @@ bool shape_supported_mixed_pp(int R, int NW, int T) {
 
 cudaError_t launch_prep_samples(const Params &P, int T, float *prep, cudaStream_t st) {
   if (P.n_particles == 0) return cudaSuccess;
-  dim3 grd(8, grid_y(P.n_particles));
+  // 256 samples per block up to 64 blocks per particle: one long trajectory has to spread over the SMs
+  const int64_t per = P.n_samples_total / P.n_particles / 256;
+  dim3 grd(static_cast<unsigned>(per < 8 ? 8 : per > 64 ? 64 : per), grid_y(P.n_particles));
   k_prep_samples<<<grd, 256, 0, st>>>(P, T, prep);
   return cudaGetLastError();
 }

@@ -78,23 +78,25 @@ __global__ void k_validate(const Params P, const double *d_omega, int need_domeg
 }
 
 // Combine partials into the cube, tile-transposed: part layout [chunk][..][j][i] (i fastest),
-// cube layout [i][j] (j fastest). Block = 32 x 8 threads over a 32 x 32 tile.
+// cube layout [i][j] (j fastest). Block = 32 x 8 threads over a tile of 32 energies x 8 directions: a
+// small grid is bound by the latency of a thread's walk over the chunks, so a thread has one bin (with
+// 32 x 32 tiles 32 blocks took 106 us for 128 x 256 bins of 32 pieces).
 template <bool AMP, int NC>
 __global__ void k_finalize(const Params P, double *cube_new, double *out_cube, int accumulate,
                            int *dev_status) {
-  __shared__ double tile[32][33];
+  __shared__ double tile[8][33];
   const int st = *reinterpret_cast<volatile int *>(P.status);
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0 && st != 0)
     atomicCAS(dev_status, 0, st);
   if (st != 0) return;  // leave the outputs untouched
   const int64_t i0 = static_cast<int64_t>(blockIdx.x) * 32;  // energy tile
   const double pref = kAlpha / (4.0 * kPi * kPi);
-  const int64_t n_jt = (P.n_angles + 31) / 32;
+  const int64_t n_jt = (P.n_angles + 7) / 8;
   for (int64_t jt = blockIdx.y; jt < n_jt; jt += gridDim.y) {  // direction tiles
-  const int64_t j0 = jt * 32;
-  // read phase: thread (x, y) reads i = i0 + x, j = j0 + y + 8k
-  for (int kk = 0; kk < 32; kk += 8) {
-    const int64_t i = i0 + threadIdx.x, j = j0 + threadIdx.y + kk;
+  const int64_t j0 = jt * 8;
+  // read phase: thread (x, y) reads i = i0 + x, j = j0 + y
+  {
+    const int64_t i = i0 + threadIdx.x, j = j0 + threadIdx.y;
     double v = 0.0;
     if (i < P.n_omega && j < P.n_angles) {
       if (!AMP) {
@@ -105,6 +107,7 @@ __global__ void k_finalize(const Params P, double *cube_new, double *out_cube, i
           double a[NC];
 #pragma unroll
           for (int c = 0; c < NC; ++c) a[c] = 0.0;
+#pragma unroll 4
           for (int q = 0; q < P.n_q; ++q) {
             const int64_t ch = p * P.n_q + q;
 #pragma unroll
@@ -130,14 +133,15 @@ __global__ void k_finalize(const Params P, double *cube_new, double *out_cube, i
         }
       }
     }
-    tile[threadIdx.y + kk][threadIdx.x] = pref * v;
+    tile[threadIdx.y][threadIdx.x] = pref * v;
   }
   __syncthreads();
-  // write phase: thread (x, y) writes j = j0 + x, i = i0 + y + 8k
-  for (int kk = 0; kk < 32; kk += 8) {
-    const int64_t j = j0 + threadIdx.x, i = i0 + threadIdx.y + kk;
+  // write phase: eight consecutive directions of an energy per eight threads
+  {
+    const int t = threadIdx.y * 32 + threadIdx.x;
+    const int64_t j = j0 + (t & 7), i = i0 + (t >> 3);
     if (i < P.n_omega && j < P.n_angles) {
-      const double v = tile[threadIdx.x][threadIdx.y + kk];
+      const double v = tile[t & 7][t >> 3];
       const int64_t e = i * P.n_angles + j;
       cube_new[e] = v;
       if (out_cube) out_cube[e] = accumulate ? out_cube[e] + v : v;
@@ -340,7 +344,7 @@ cudaError_t launch_finalize(const Params &P, double *cube_new, double *out_cube,
   int *ds = device_status_word(&e);
   if (!ds) return e;
   dim3 blk(32, 8);
-  dim3 grd(static_cast<unsigned>((P.n_omega + 31) / 32), grid_y((P.n_angles + 31) / 32));
+  dim3 grd(static_cast<unsigned>((P.n_omega + 31) / 32), grid_y((P.n_angles + 7) / 8));
   if (grd.x == 0 || grd.y == 0) return cudaSuccess;
   if (!P.amp_mode)
     k_finalize<false, 6><<<grd, blk, 0, st>>>(P, cube_new, out_cube, accumulate, ds);
@@ -354,7 +358,7 @@ cudaError_t launch_finalize(const Params &P, double *cube_new, double *out_cube,
 cudaError_t launch_finalize_status(const Params &P, double *cube_new, double *out_cube, int accumulate,
                                    int *publish_status, cudaStream_t st) {
   dim3 blk(32, 8);
-  dim3 grd(static_cast<unsigned>((P.n_omega + 31) / 32), grid_y((P.n_angles + 31) / 32));
+  dim3 grd(static_cast<unsigned>((P.n_omega + 31) / 32), grid_y((P.n_angles + 7) / 8));
   if (grd.x == 0 || grd.y == 0) return cudaSuccess;
   if (P.amp_mode) return cudaErrorInvalidValue;
   k_finalize<false, 6><<<grd, blk, 0, st>>>(P, cube_new, out_cube, accumulate, publish_status);
