@@ -278,7 +278,7 @@ __global__ void k_channel(const Chan C, const Planar P, int64_t n_particles, con
 // ------------------------------------------------------------------------------------
 struct Axial {
   int nt, nb, K, el;
-  double Lx, Ly;
+  double Lx, Ly, inv_Lx, inv_Ly;
   double sx[8], sy[8];
   double fk[kMaxTerms];  // q (2 e^2 a0 / d) (a_i / C_i) (2 / C_i)
   double ck[kMaxTerms];  // 1 / C_i
@@ -381,6 +381,64 @@ __device__ __forceinline__ State deriv_axial(const Chan &C, const Axial &A, doub
   return d;
 }
 
+// ------------------------------------------------------------------------------------
+// Pieces of the lane-group kernels: FP64 divisions and square roots cost some
+// ten dependent instructions each, and a step is one dependent chain.
+// ------------------------------------------------------------------------------------
+// 1 / v for normal v: one cubic step from the hardware's 20-bit reciprocal
+__device__ __forceinline__ double rcp_fast(double v) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
+  const double e = fma(-v, r, 1.0);
+  return fma(fma(e, e, e), r, r);
+}
+
+// sqrt(a) and 1 / sqrt(a) for normal a > 0: one cubic step from the hardware's reciprocal root, and a
+// Newton correction of the root; any other a takes sqrt and a division
+__device__ __forceinline__ double sqrt_fast(double a, double &inv) {
+  if (!(a > 1e-290)) {
+    const double r = sqrt(a);
+    inv = 1.0 / r;
+    return r;
+  }
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const double e = fma(-(a * y), y, 1.0);
+  y = fma(y * e, fma(e, 0.375, 0.5), y);
+  inv = y;
+  const double r = a * y;
+  return fma(0.5 * y, fma(-r, r, a), r);
+}
+
+// What a stage needs of the energy: g, 1/E, 1/g^2 and the energy part of the longitudinal velocity
+// (1/g0^2 - 1/g^2 and 1 - 1/g^2)
+struct EnergyPart {
+  double g, inv_E, ig2, d_inv, one;
+};
+__device__ __forceinline__ EnergyPart energy_part(double E, double inv_mass, double g0, double ig02) {
+  EnergyPart e;
+  e.g = E * inv_mass;
+  e.inv_E = rcp_fast(E);
+  const double ig = rcp_fast(e.g);
+  e.ig2 = ig * ig;
+  e.d_inv = ((e.g - g0) * (e.g + g0)) * (e.ig2 * ig02);
+  e.one = 1.0 - e.ig2;
+  return e;
+}
+
+// v_z - beta0 (see dvz_of) and 1 / v_z
+__device__ __forceinline__ double dvz_fast(const EnergyPart &e, double q0, double beta0, double vp2, double &inv_vz) {
+  const double vz = sqrt_fast(e.one - vp2, inv_vz);
+  return (e.d_inv - vp2 - q0) * rcp_fast(vz + beta0);
+}
+
+// Electron part of the scattering variance per (1/2) dt pi r0^2 n_el
+__device__ __forceinline__ double electron_bracket(double lk, const EnergyPart &e) {
+  const double g2 = e.g * e.g;
+  const double br = fmax(log(lk * g2 * e.one) - e.one, 0.0);
+  return br * e.ig2 * rcp_fast(e.one * e.one);
+}
+
 // Small ensembles: one particle per group of kGroup lanes. The lanes share the force evaluation
 // (each takes some of the (basis string, term) pairs, the partial forces are summed by a butterfly
 // of shuffles within the group) and keep identical copies of the state, so a step's exponentials
@@ -402,17 +460,48 @@ __device__ __forceinline__ double group_sum(double v, unsigned mask) {
   return __shfl_sync(mask, v, 0, kGroup);
 }
 
+// axis_sums with two exponentials instead of three: the ratios of the first images above and below
+// multiply to q. Where k L^2 > 150 every image but the nearest is below e^{-37.5} = 5e-17 of the
+// Gaussian's height and is left out (there the quotient would also lose its range).
+__device__ __forceinline__ void axis_sums_fast(double u0, double L, int K, double k, double q, double &s1, double &s0) {
+  const int i0 = u0 > 0.5 * L ? 1 : (u0 < -0.5 * L ? -1 : 0);
+  const double r = fma(-static_cast<double>(i0), L, u0);
+  const double E0 = exp(-(r * r) * k);
+  s1 = r * E0;
+  s0 = E0;
+  if (k * (L * L) > 150.0) return;
+  const double up = exp(k * (2.0 * r * L - L * L));
+  double E = E0, rho = up, u = r;
+  for (int m = 0; m < K - i0; ++m) {  // images i0 + 1 .. K at r - m L
+    E *= rho;
+    rho *= q;
+    u -= L;
+    s1 = fma(u, E, s1);
+    s0 += E;
+  }
+  E = E0;
+  rho = q * rcp_fast(up);
+  u = r;
+  for (int m = 0; m < K + i0; ++m) {  // images i0 - 1 .. -K at r + m L
+    E *= rho;
+    rho *= q;
+    u += L;
+    s1 = fma(u, E, s1);
+    s0 += E;
+  }
+}
+
 __device__ __forceinline__ void axial_force_group(const Axial &A, double x, double y, int gl, unsigned mask,
                                                   double &Fx, double &Fy) {
-  const double cx = floor(x / A.Lx), cy = floor(y / A.Ly);
+  const double cx = floor(x * A.inv_Lx), cy = floor(y * A.inv_Ly);
   double fx = 0.0, fy = 0.0;
   for (int q = gl; q < A.nb * A.nt; q += kGroup) {
     const int b = q / A.nt, t = q - b * A.nt;
     const double ux = x - (cx * A.Lx + A.sx[b]);
     const double uy = y - (cy * A.Ly + A.sy[b]);
     double sx1, sx0, sy1, sy0;
-    axis_sums(ux, A.Lx, A.K, A.ck[t], A.qx[t], sx1, sx0);
-    axis_sums(uy, A.Ly, A.K, A.ck[t], A.qy[t], sy1, sy0);
+    axis_sums_fast(ux, A.Lx, A.K, A.ck[t], A.qx[t], sx1, sx0);
+    axis_sums_fast(uy, A.Ly, A.K, A.ck[t], A.qy[t], sy1, sy0);
     fx += A.fk[t] * (sx1 * sy0);
     fy += A.fk[t] * (sx0 * sy1);
   }
@@ -422,18 +511,18 @@ __device__ __forceinline__ void axial_force_group(const Axial &A, double x, doub
 
 __device__ __forceinline__ void axial_densities_group(const Axial &A, double x, double y, int gl, unsigned mask,
                                                       double &n_nuc, double &n_el) {
-  const double cx = floor(x / A.Lx), cy = floor(y / A.Ly);
+  const double cx = floor(x * A.inv_Lx), cy = floor(y * A.inv_Ly);
   double nn = 0.0, ne = 0.0, s1, sx0, sy0;
   for (int b = gl; b < A.nb; b += kGroup) {
-    axis_sums(x - (cx * A.Lx + A.sx[b]), A.Lx, A.K, A.inv_rho2, A.rqx, s1, sx0);
-    axis_sums(y - (cy * A.Ly + A.sy[b]), A.Ly, A.K, A.inv_rho2, A.rqy, s1, sy0);
+    axis_sums_fast(x - (cx * A.Lx + A.sx[b]), A.Lx, A.K, A.inv_rho2, A.rqx, s1, sx0);
+    axis_sums_fast(y - (cy * A.Ly + A.sy[b]), A.Ly, A.K, A.inv_rho2, A.rqy, s1, sy0);
     nn += sx0 * sy0;
   }
   if (A.el) {
     for (int q = gl; q < A.nb * A.nt; q += kGroup) {
       const int b = q / A.nt, t = q - b * A.nt;
-      axis_sums(x - (cx * A.Lx + A.sx[b]), A.Lx, A.K, A.eck[t], A.eqx[t], s1, sx0);
-      axis_sums(y - (cy * A.Ly + A.sy[b]), A.Ly, A.K, A.eck[t], A.eqy[t], s1, sy0);
+      axis_sums_fast(x - (cx * A.Lx + A.sx[b]), A.Lx, A.K, A.eck[t], A.eqx[t], s1, sx0);
+      axis_sums_fast(y - (cy * A.Ly + A.sy[b]), A.Ly, A.K, A.eck[t], A.eqy[t], s1, sy0);
       ne += A.ek[t] * (sx0 * sy0);
     }
   }
@@ -441,24 +530,20 @@ __device__ __forceinline__ void axial_densities_group(const Axial &A, double x, 
   n_el = (A.el ? group_sum(ne, mask) : 0.0) + A.ecx * n_nuc;
 }
 
-__device__ __forceinline__ State deriv_axial_group(const Chan &C, const Axial &A, double g0, double q0, double beta0,
-                                                   const State &s, int gl, unsigned mask) {
-  const double g = s.E / C.mass;
-  const double vp2 = s.vx * s.vx + s.vy * s.vy;
-  double vz;
-  const double dvz = dvz_of(g, g0, q0, beta0, vp2, vz);
-  double Fx, Fy;
-  axial_force_group(A, s.x, s.y, gl, mask, Fx, Fy);
-  State d;
-  d.x = s.vx;
-  d.y = s.vy;
-  d.vx = Fx / s.E;
-  d.vy = Fy / s.E;
-  d.dz = dvz;
-  d.E = C.ll ? C.ll_k * (g * g) * (Fx * Fx + Fy * Fy) : 0.0;
-  return d;
+// time derivatives of one RK4 stage: (v_x, v_y, dz, E)
+struct AxialStage {
+  double ax, ay, dz, dE;
+};
+__device__ __forceinline__ AxialStage axial_stage(const Chan &C, const EnergyPart &e, double q0, double beta0,
+                                                  double vx, double vy, double Fx, double Fy) {
+  double iv;
+  const double dz = dvz_fast(e, q0, beta0, fma(vx, vx, vy * vy), iv);
+  return AxialStage{Fx * e.inv_E, Fy * e.inv_E, dz, C.ll ? C.ll_k * (e.g * e.g) * fma(Fx, Fx, Fy * Fy) : 0.0};
 }
 
+// The record's force is the first stage's, so a step evaluates the force four times; the divisions
+// and roots of the kinematics are the short forms above, and every lane draws the kick of one of the
+// next kGroup steps.
 __global__ void k_axial_group(const Chan C, const Axial A, int64_t n_particles, const int64_t *__restrict__ offsets,
                               int64_t n_total, const double *__restrict__ energy, const double *__restrict__ x0,
                               const double *__restrict__ y0, const double *__restrict__ thx0,
@@ -466,6 +551,7 @@ __global__ void k_axial_group(const Chan C, const Axial A, int64_t n_particles, 
                               uint64_t seed, double *__restrict__ out, double *__restrict__ e_out, int *dev_status) {
   const int gl = threadIdx.x & (kGroup - 1);
   const unsigned mask = 0xFFFFu << (threadIdx.x & 16);
+  const double inv_mass = 1.0 / C.mass, inv_dt = 1.0 / dt, h6 = dt / 6.0;
   const int64_t groups = static_cast<int64_t>(gridDim.x) * (blockDim.x / kGroup);
   for (int64_t p = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) / kGroup; p < n_particles;
        p += groups) {
@@ -477,72 +563,84 @@ __global__ void k_axial_group(const Chan C, const Axial A, int64_t n_particles, 
       continue;
     }
     const uint64_t pid = ids ? static_cast<uint64_t>(ids[p]) : static_cast<uint64_t>(p);
-    const double g0 = E0 / C.mass;
-    const double beta0 = 1.0 - 1.0 / (2.0 * g0 * g0);
-    const double q0 = 1.0 / (4.0 * (g0 * g0) * (g0 * g0));
-    State s{x0[p], y0 ? y0[p] : 0.0, thx0[p], thy0 ? thy0[p] : 0.0, 0.0, E0};
-    double kx = 0.0, ky = 0.0;
+    const double g0 = E0 * inv_mass, ig02 = 1.0 / (g0 * g0);
+    const double beta0 = 1.0 - 0.5 * ig02, q0 = 0.25 * (ig02 * ig02);
+    double x = x0[p], y = y0 ? y0[p] : 0.0, vx = thx0[p], vy = thy0 ? thy0[p] : 0.0, dz = 0.0, E = E0;
+    EnergyPart ep = energy_part(E, inv_mass, g0, ig02);
+    double br = A.el ? electron_bracket(A.lk, ep) : 0.0;
+    double kx = 0.0, ky = 0.0, z0 = 0.0, z1 = 0.0;
     double *rec = out + off * kRec;
     for (int64_t k = 0; k < L; ++k, rec += kRec) {
-      const double g = s.E / C.mass;
-      const double vp2 = s.vx * s.vx + s.vy * s.vy;
-      double vz;
-      const double dvz = dvz_of(g, g0, q0, beta0, vp2, vz);
-      double Fx, Fy;
-      axial_force_group(A, s.x, s.y, gl, mask, Fx, Fy);
-      const double ax = Fx / s.E + kx, ay = Fy / s.E + ky;
-      const double gdot = C.ll ? C.ll_k * (g * g) * (Fx * Fx + Fy * Fy) / C.mass : 0.0;
+      double Fx, Fy, inv_vz;
+      axial_force_group(A, x, y, gl, mask, Fx, Fy);
+      const double vp2 = fma(vx, vx, vy * vy);
+      const double dvz = dvz_fast(ep, q0, beta0, vp2, inv_vz);
+      const AxialStage k1{Fx * ep.inv_E, Fy * ep.inv_E, dvz,
+                          C.ll ? C.ll_k * (ep.g * ep.g) * fma(Fx, Fx, Fy * Fy) : 0.0};
+      const double ax = k1.ax + kx, ay = k1.ay + ky;
       // every lane holds the record; lane f writes field f
       double v = 0.0;
       switch (gl) {
         case F_T: v = static_cast<double>(k) * dt; break;
-        case F_X: v = s.x; break;
-        case F_Y: v = s.y; break;
-        case F_DZ: v = s.dz; break;
-        case F_VX: v = s.vx; break;
-        case F_VY: v = s.vy; break;
+        case F_X: v = x; break;
+        case F_Y: v = y; break;
+        case F_DZ: v = dz; break;
+        case F_VX: v = vx; break;
+        case F_VY: v = vy; break;
         case F_DVZ: v = dvz; break;
         case F_AX: v = ax; break;
         case F_AY: v = ay; break;
-        case F_AZ: v = (gdot / (g * g * g) - (s.vx * ax + s.vy * ay)) / vz; break;
+        case F_AZ: {
+          const double ig = ep.g * ep.ig2;
+          v = fma(k1.dE * inv_mass, ig * ep.ig2, -fma(vx, ax, vy * ay)) * inv_vz;
+          break;
+        }
         default: break;
       }
       if (gl < kRec) rec[gl] = v;
-      if (e_out && gl == 0) e_out[off + k] = s.E;
+      if (e_out && gl == 0) e_out[off + k] = E;
       kx = ky = 0.0;
       if (k == L - 1) break;
-      const State k1 = deriv_axial_group(C, A, g0, q0, beta0, s, gl, mask);
-      const State k2 = deriv_axial_group(C, A, g0, q0, beta0, axpy(s, 0.5 * dt, k1), gl, mask);
-      const State k3 = deriv_axial_group(C, A, g0, q0, beta0, axpy(s, 0.5 * dt, k2), gl, mask);
-      const State k4 = deriv_axial_group(C, A, g0, q0, beta0, axpy(s, dt, k3), gl, mask);
-      const double h6 = dt / 6.0;
-      s.x += h6 * (k1.x + 2.0 * k2.x + 2.0 * k3.x + k4.x);
-      s.y += h6 * (k1.y + 2.0 * k2.y + 2.0 * k3.y + k4.y);
-      s.vx += h6 * (k1.vx + 2.0 * k2.vx + 2.0 * k3.vx + k4.vx);
-      s.vy += h6 * (k1.vy + 2.0 * k2.vy + 2.0 * k3.vy + k4.vy);
-      s.dz += h6 * (k1.dz + 2.0 * k2.dz + 2.0 * k3.dz + k4.dz);
-      s.E += h6 * (k1.E + 2.0 * k2.E + 2.0 * k3.E + k4.E);
+      auto at = [&](double h, const AxialStage &s) {
+        return C.ll ? energy_part(fma(h, s.dE, E), inv_mass, g0, ig02) : ep;
+      };
+      const double hh = 0.5 * dt;
+      const double vx2 = fma(hh, k1.ax, vx), vy2 = fma(hh, k1.ay, vy);
+      axial_force_group(A, fma(hh, vx, x), fma(hh, vy, y), gl, mask, Fx, Fy);
+      const AxialStage k2 = axial_stage(C, at(hh, k1), q0, beta0, vx2, vy2, Fx, Fy);
+      const double vx3 = fma(hh, k2.ax, vx), vy3 = fma(hh, k2.ay, vy);
+      axial_force_group(A, fma(hh, vx2, x), fma(hh, vy2, y), gl, mask, Fx, Fy);
+      const AxialStage k3 = axial_stage(C, at(hh, k2), q0, beta0, vx3, vy3, Fx, Fy);
+      const double vx4 = fma(dt, k3.ax, vx), vy4 = fma(dt, k3.ay, vy);
+      axial_force_group(A, fma(dt, vx3, x), fma(dt, vy3, y), gl, mask, Fx, Fy);
+      const AxialStage k4 = axial_stage(C, at(dt, k3), q0, beta0, vx4, vy4, Fx, Fy);
+      x += h6 * (vx + 2.0 * vx2 + 2.0 * vx3 + vx4);
+      y += h6 * (vy + 2.0 * vy2 + 2.0 * vy3 + vy4);
+      vx += h6 * (k1.ax + 2.0 * k2.ax + 2.0 * k3.ax + k4.ax);
+      vy += h6 * (k1.ay + 2.0 * k2.ay + 2.0 * k3.ay + k4.ay);
+      dz += h6 * (k1.dz + 2.0 * k2.dz + 2.0 * k3.dz + k4.dz);
+      if (C.ll) {
+        E += h6 * (k1.dE + 2.0 * k2.dE + 2.0 * k3.dE + k4.dE);
+        ep = energy_part(E, inv_mass, g0, ig02);
+        if (A.el) br = electron_bracket(A.lk, ep);
+      }
       if (C.ms) {
-        const double E = s.E;
         double n_nuc, n_el;
-        axial_densities_group(A, s.x, s.y, gl, mask, n_nuc, n_el);
-        double var = C.var_k / (E * E) * n_nuc;
-        if (A.el) {
-          const double ge = E / C.mass, b2 = 1.0 - 1.0 / (ge * ge);
-          const double br = fmax(log(A.lk * (ge * ge) * b2) - b2, 0.0);
-          var += n_el * (br / ((ge * ge) * (b2 * b2)));
-        }
-        double z0, z1;
-        kick_normals(seed, pid, static_cast<uint64_t>(k), z0, z1);
+        axial_densities_group(A, x, y, gl, mask, n_nuc, n_el);
+        const int lane_k = static_cast<int>(k % kGroup);
+        if (lane_k == 0) kick_normals(seed, pid, static_cast<uint64_t>(k + gl), z0, z1);
+        double var = C.var_k * (ep.inv_E * ep.inv_E) * n_nuc;
+        if (A.el) var = fma(n_el, br, var);
         const double sd = sqrt(var);
-        const double dthx = sd * z0, dthy = sd * z1;
-        kx = dthx / dt;
-        ky = dthy / dt;
-        s.vx += dthx;
-        s.vy += dthy;
+        const double dthx = sd * __shfl_sync(mask, z0, lane_k, kGroup), dthy = sd * __shfl_sync(mask, z1, lane_k, kGroup);
+        kx = dthx * inv_dt;
+        ky = dthy * inv_dt;
+        vx += dthx;
+        vy += dthy;
         if (C.ms_loss) {
-          const double gk = E / C.mass;
-          s.E = E - C.loss_k * (gk * gk * gk) * (dthx * dthx + dthy * dthy);
+          E -= C.loss_k * (ep.g * ep.g * ep.g) * (dthx * dthx + dthy * dthy);
+          ep = energy_part(E, inv_mass, g0, ig02);
+          if (A.el) br = electron_bracket(A.lk, ep);
         }
       }
     }
@@ -1464,8 +1562,8 @@ int launch_trajectories(const rad_channel *ch, const rad_planar_potential *pot, 
           M, P32, n_particles, offsets, n_samples_total, energy_eV, x0, thx0, thy0, particle_ids, seed, out,
           energy_out, ds);
   } else if (pot && n_particles < kPGroupBelow) {  // lane groups share each particle's force evaluation
-    const int64_t ggrid = (n_particles * kPGroup + 127) / 128;
-    k_channel_group<<<static_cast<unsigned>(ggrid), 128, 0, st>>>(C, P, n_particles, offsets, n_samples_total,
+    const int64_t ggrid = (n_particles * kPGroup + 31) / 32;
+    k_channel_group<<<static_cast<unsigned>(ggrid), 32, 0, st>>>(C, P, n_particles, offsets, n_samples_total,
                                                                  energy_eV, x0, thx0, thy0, particle_ids, dt, seed,
                                                                  out, energy_out, ds);
   } else if (pot) {
@@ -1500,6 +1598,8 @@ int make_axial(const rad_channel *ch, const rad_axial_potential *pot, double dt,
   A.el = el ? 1 : 0;
   A.Lx = Lt.cell_x;
   A.Ly = Lt.cell_y;
+  A.inv_Lx = 1.0 / A.Lx;
+  A.inv_Ly = 1.0 / A.Ly;
   for (int b = 0; b < A.nb; ++b) {
     if (!isfinite(Lt.sx[b]) || !isfinite(Lt.sy[b])) return RAD_EINVAL;
     A.sx[b] = Lt.sx[b];
@@ -1567,7 +1667,7 @@ int launch_axial(const rad_channel *ch, const rad_axial_potential *pot, int64_t 
   C.ll = (ch->flags & RAD_TRAJ_LL) != 0;
   C.ms_loss = (ch->flags & RAD_TRAJ_MS_LOSS) != 0;
   if (n_particles < kGroupBelow) {  // lane groups share each particle's force evaluation
-    const int block = 128;
+    const int block = 32;  // one-warp blocks: two particles each, spread evenly over the SMs
     const int64_t grid = (n_particles * kGroup + block - 1) / block;
     k_axial_group<<<static_cast<unsigned>(grid), block, 0, static_cast<cudaStream_t>(stream)>>>(
         C, A, n_particles, offsets, n_samples_total, energy_eV, x0, y0, thx0, thy0, particle_ids, dt, seed, out,
