@@ -382,7 +382,7 @@ __device__ __forceinline__ State deriv_axial(const Chan &C, const Axial &A, doub
 }
 
 // ------------------------------------------------------------------------------------
-// Pieces of the lane-group kernels: FP64 divisions and square roots cost some
+// Pieces of the tabulated and of the lane-group kernels: FP64 divisions and square roots cost some
 // ten dependent instructions each, and a step is one dependent chain.
 // ------------------------------------------------------------------------------------
 // 1 / v for normal v: one cubic step from the hardware's 20-bit reciprocal
@@ -641,6 +641,203 @@ __global__ void k_axial_group(const Chan C, const Axial A, int64_t n_particles, 
           E -= C.loss_k * (ep.g * ep.g * ep.g) * (dthx * dthx + dthy * dthy);
           ep = energy_part(E, inv_mass, g0, ig02);
           if (A.el) br = electron_bracket(A.lk, ep);
+        }
+      }
+    }
+  }
+}
+
+// ------------------------------------------------------------------------------------
+// Doyle-Turner planar potential from a table. Force and densities are functions of the position
+// within one cell [0, d_p) only, so every block expands them once, at the centres of kTabI equal
+// intervals, in Taylor polynomials of degree kTabDeg (Gaussians: g = e^{-k (r + s)^2} has
+// (n+1) g_{n+1} = -2 k r g_n - 2 k g_{n-1}), and a stage costs one polynomial instead of three
+// exponentials per term of the fit. With intervals of at most a tenth of the narrowest Gaussian's
+// sqrt(C) (tab_fits) the first dropped term is below 1e-16 of that Gaussian. The table takes about
+// 0.2 ms a block, a step about 8 us.
+//
+// G lanes hold one particle: G = 4 for small ensembles, where the dependent chain of a step bounds
+// the time: lanes 0 to 2 evaluate force, nuclear and electron density at once, each lane draws the
+// kicks of one of the next four steps, and the lanes share the record's stores. G = 1 from about two
+// warps per SM on (kTabGroupBelow), where the FP64 pipe is busy and copies of the state would cost.
+// ------------------------------------------------------------------------------------
+constexpr int kTabI = 256, kTabDeg = 11, kTabC = kTabDeg + 1;
+constexpr int kTabThreads = 128;
+constexpr int64_t kTabGroupBelow = 2432;
+constexpr size_t kTabBytes = sizeof(double) * 3 * kTabI * kTabC;
+
+// The polynomials resolve the fit: intervals of at most a tenth of the narrowest Gaussian.
+inline bool tab_fits(const Planar &P, const Chan &C) {
+  const double h = C.d_p / kTabI;
+  double k = C.ms ? C.inv_rho2 : 0.0;
+  for (int i = 0; i < P.nt; ++i) {
+    k = fmax(k, P.ck[i]);
+    if (P.el) k = fmax(k, P.eck[i]);
+  }
+  return h * h * k <= 0.0101;
+}
+
+__device__ __forceinline__ void tab_add(double (&c)[kTabC], double amp, double k, double r, double h, bool times_r) {
+  const double e = k * r * r;
+  if (e > 90.0) return;  // below 1e-39 of the Gaussian's height over the whole interval
+  double g0 = amp * exp(-e);
+  const double a = -2.0 * k * r * h, b = -2.0 * k * h * h;
+  double gm = 0.0;  // g_{n-1}
+#pragma unroll
+  for (int n = 0; n < kTabC; ++n) {
+    c[n] += times_r ? fma(r, g0, h * gm) : g0;
+    const double g1 = fma(a, g0, b * gm) * (1.0 / (n + 1));
+    gm = g0;
+    g0 = g1;
+  }
+}
+
+// table: 0 force, 1 n(x)/N, 2 (1/2) dt pi r0^2 n_el
+__device__ void tab_build(const Chan &C, const Planar &P, double *tab) {
+  const double h = 0.5 * C.d_p / kTabI;
+  const int n_tab = C.ms ? (P.el ? 3 : 2) : 1;
+  for (int u = threadIdx.x; u < n_tab * kTabI; u += kTabThreads) {
+    const int t = u / kTabI, i = u - t * kTabI;
+    const double x = (2 * i + 1) * h;
+    double c[kTabC];
+#pragma unroll
+    for (int n = 0; n < kTabC; ++n) c[n] = 0.0;
+    if (t != 0)  // nuclear density: the two nearest planes
+      for (int j = 0; j < 2; ++j) tab_add(c, t == 1 ? C.dens_pref : P.ecx * C.dens_pref, C.inv_rho2, x - j * C.d_p, h, false);
+    if (t != 1)
+      for (int j = 1 - P.K; j <= P.K; ++j)
+        for (int m = 0; m < P.nt; ++m)
+          tab_add(c, t ? P.ek[m] : P.fk[m], t ? P.eck[m] : P.ck[m], x - j * C.d_p, h, t == 0);
+#pragma unroll
+    for (int n = 0; n < kTabC; ++n) tab[u * kTabC + n] = c[n];
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ double tab_eval(const Chan &C, const double *tab, double x) {
+  const double xi = fma(-floor(x * C.inv_d), C.d_p, x);
+  const double t = xi * (C.inv_d * kTabI);
+  int i = static_cast<int>(t);
+  i = i < 0 ? 0 : i > kTabI - 1 ? kTabI - 1 : i;
+  const double s = fma(2.0, t - i, -1.0);
+  const double2 *c = reinterpret_cast<const double2 *>(tab + i * kTabC);
+  const double s2 = s * s, s4 = s2 * s2;
+  double q[kTabC / 2];
+#pragma unroll
+  for (int n = 0; n < kTabC / 2; ++n) {
+    const double2 v = c[n];
+    q[n] = fma(v.y, s, v.x);
+  }
+  // 1, s^2, .., s^10 by pairs: a chain of four
+  const double lo = fma(q[1], s2, q[0]), mid = fma(q[3], s2, q[2]), hi = fma(q[5], s2, q[4]);
+  return fma(fma(hi, s4, mid), s4, lo);
+}
+
+struct Stage {
+  double ax, dz, dE;  // dv_x/dt, d(dz)/dt, dE/dt
+};
+
+template <int G>
+__global__ void __launch_bounds__(kTabThreads) k_channel_tab(
+    const Chan C, const Planar P, int64_t n_particles, const int64_t *__restrict__ offsets, int64_t n_total,
+    const double *__restrict__ energy, const double *__restrict__ x0, const double *__restrict__ thx0,
+    const double *__restrict__ thy0, const int64_t *__restrict__ ids, double dt, uint64_t seed,
+    double *__restrict__ out, double *__restrict__ e_out, int *dev_status) {
+  static_assert(G == 1 || G == 4, "lanes per particle");
+  extern __shared__ __align__(16) double tab[];
+  tab_build(C, P, tab);
+  const int gl = threadIdx.x % G;
+  const unsigned mask = G == 1 ? 1u << (threadIdx.x & 31) : 0xFu << (threadIdx.x & 28);
+  const double inv_mass = 1.0 / C.mass, inv_dt = 1.0 / dt, h6 = dt / 6.0;
+  // this lane's table in the joint evaluation
+  const double *mine = tab + ((gl == 1 && C.ms) ? kTabI * kTabC : (gl == 2 && P.el) ? 2 * kTabI * kTabC : 0);
+  auto from = [&](double v, int l) { return G == 1 ? v : __shfl_sync(mask, v, l, G); };
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * (kTabThreads / G);
+  for (int64_t p = blockIdx.x + static_cast<int64_t>(threadIdx.x / G) * gridDim.x; p < n_particles; p += stride) {
+    const int64_t off = offsets[p], L = offsets[p + 1] - off;
+    const double E0 = energy[p];
+    if (off < 0 || L < 1 || off + L > n_total || !(E0 > C.mass) || !isfinite(E0) || !isfinite(x0[p]) ||
+        !isfinite(thx0[p]) || (thy0 && !isfinite(thy0[p]))) {
+      if (gl == 0) atomicCAS(dev_status, 0, RAD_EDATA);
+      continue;
+    }
+    const uint64_t pid = ids ? static_cast<uint64_t>(ids[p]) : static_cast<uint64_t>(p);
+    const double g0 = E0 * inv_mass, ig02 = 1.0 / (g0 * g0);
+    const double beta0 = 1.0 - 0.5 * ig02, q0 = 0.25 * (ig02 * ig02);
+    double x = x0[p], y = 0.0, vx = thx0[p], vy = thy0 ? thy0[p] : 0.0, dz = 0.0, E = E0;
+    EnergyPart ep = energy_part(E, inv_mass, g0, ig02);
+    double br = P.el ? electron_bracket(P.lk, ep) : 0.0;
+    double kx = 0.0, ky = 0.0, z0 = 0.0, z1 = 0.0;
+    double F = tab_eval(C, tab, x);
+    double *rec = out + off * kRec;
+    auto stage = [&](const EnergyPart &e, double f, double vp2) {
+      double iv;
+      return Stage{f * e.inv_E, dvz_fast(e, q0, beta0, vp2, iv), C.ll ? C.ll_k * (e.g * e.g) * (f * f) : 0.0};
+    };
+    for (int64_t k = 0; k < L; ++k, rec += kRec) {
+      const double vy2 = vy * vy, vp2 = fma(vx, vx, vy2);
+      double inv_vz;
+      const double dvz = dvz_fast(ep, q0, beta0, vp2, inv_vz);
+      const Stage k1{F * ep.inv_E, dvz, C.ll ? C.ll_k * (ep.g * ep.g) * (F * F) : 0.0};
+      const double ax = k1.ax + kx, ay = ky;
+      const double ig = ep.g * ep.ig2;
+      const double az = fma(k1.dE * inv_mass, ig * ep.ig2, -fma(vx, ax, vy * ay)) * inv_vz;
+      const double t = static_cast<double>(k) * dt;
+      if (G == 1) {
+        rec[F_T] = t;
+        rec[F_X] = x;
+        rec[F_Y] = y;
+        rec[F_DZ] = dz;
+        rec[F_VX] = vx;
+        rec[F_VY] = vy;
+        rec[F_DVZ] = dvz;
+        rec[F_AX] = ax;
+        rec[F_AY] = ay;
+        rec[F_AZ] = az;
+      } else {  // lane l writes fields l, l + 4 and, for two lanes, l + 8
+        rec[gl] = gl == 0 ? t : gl == 1 ? x : gl == 2 ? y : dz;
+        rec[gl + 4] = gl == 0 ? vx : gl == 1 ? vy : gl == 2 ? dvz : ax;
+        if (gl < 2) rec[gl + 8] = gl == 0 ? ay : az;
+      }
+      if (e_out && gl == 0) e_out[off + k] = E;
+      kx = ky = 0.0;
+      if (k == L - 1) break;
+      // RK4 step; v_y is constant within it
+      const double hh = 0.5 * dt;
+      auto at = [&](double h, const Stage &s) { return C.ll ? energy_part(fma(h, s.dE, E), inv_mass, g0, ig02) : ep; };
+      const double vx2 = fma(hh, k1.ax, vx);
+      const Stage k2 = stage(at(hh, k1), tab_eval(C, tab, fma(hh, vx, x)), fma(vx2, vx2, vy2));
+      const double vx3 = fma(hh, k2.ax, vx);
+      const Stage k3 = stage(at(hh, k2), tab_eval(C, tab, fma(hh, vx2, x)), fma(vx3, vx3, vy2));
+      const double vx4 = fma(dt, k3.ax, vx);
+      const Stage k4 = stage(at(dt, k3), tab_eval(C, tab, fma(dt, vx3, x)), fma(vx4, vx4, vy2));
+      x += h6 * (vx + 2.0 * vx2 + 2.0 * vx3 + vx4);
+      y += h6 * (6.0 * vy);
+      vx += h6 * (k1.ax + 2.0 * k2.ax + 2.0 * k3.ax + k4.ax);
+      dz += h6 * (k1.dz + 2.0 * k2.dz + 2.0 * k3.dz + k4.dz);
+      if (C.ll) {
+        E += h6 * (k1.dE + 2.0 * k2.dE + 2.0 * k3.dE + k4.dE);
+        ep = energy_part(E, inv_mass, g0, ig02);
+        if (P.el) br = electron_bracket(P.lk, ep);
+      }
+      // the force at the next record's position, and the densities of the kick there
+      const double own = tab_eval(C, mine, x);
+      F = from(own, 0);
+      if (C.ms) {
+        const int lane_k = static_cast<int>(k % G);
+        if (lane_k == 0) kick_normals(seed, pid, static_cast<uint64_t>(k + gl), z0, z1);
+        double var = C.var_k * (ep.inv_E * ep.inv_E) * (G == 1 ? tab_eval(C, tab + kTabI * kTabC, x) : from(own, 1));
+        if (P.el) var = fma(G == 1 ? tab_eval(C, tab + 2 * kTabI * kTabC, x) : from(own, 2), br, var);
+        const double sd = sqrt(var);
+        const double dthx = sd * from(z0, lane_k), dthy = sd * from(z1, lane_k);
+        kx = dthx * inv_dt;
+        ky = dthy * inv_dt;
+        vx += dthx;
+        vy += dthy;
+        if (C.ms_loss) {
+          E -= C.loss_k * (ep.g * ep.g * ep.g) * (dthx * dthx + dthy * dthy);
+          ep = energy_part(E, inv_mass, g0, ig02);
+          if (P.el) br = electron_bracket(P.lk, ep);
         }
       }
     }
@@ -1561,6 +1758,18 @@ int launch_trajectories(const rad_channel *ch, const rad_planar_potential *pot, 
       k_channel_mixed<false><<<static_cast<unsigned>(grid), block, 0, st>>>(
           M, P32, n_particles, offsets, n_samples_total, energy_eV, x0, thx0, thy0, particle_ids, seed, out,
           energy_out, ds);
+  } else if (pot && tab_fits(P, C)) {
+    const bool four = n_particles < kTabGroupBelow;
+    auto kern = four ? k_channel_tab<4> : k_channel_tab<1>;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kTabBytes));
+    if (e != cudaSuccess) return cuda_status(e);
+    // one block per SM as long as its 128 threads hold the particles, else up to three
+    const int64_t per_block = four ? kTabThreads / 4 : kTabThreads;
+    const int64_t blocks = (n_particles + per_block - 1) / per_block;
+    const int64_t tgrid = n_particles < 152 ? n_particles : blocks <= 152 ? 152 : blocks < 456 ? blocks : 456;
+    kern<<<static_cast<unsigned>(tgrid), kTabThreads, kTabBytes, st>>>(C, P, n_particles, offsets, n_samples_total,
+                                                                      energy_eV, x0, thx0, thy0, particle_ids, dt,
+                                                                      seed, out, energy_out, ds);
   } else if (pot && n_particles < kPGroupBelow) {  // lane groups share each particle's force evaluation
     const int64_t ggrid = (n_particles * kPGroup + 31) / 32;
     k_channel_group<<<static_cast<unsigned>(ggrid), 32, 0, st>>>(C, P, n_particles, offsets, n_samples_total,
