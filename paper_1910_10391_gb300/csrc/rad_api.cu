@@ -49,6 +49,7 @@ struct rad_plan_s {
   Choice choice{};
   LaunchShape shape{};
   int n_wt = 0, n_nt = 0, amp_mode = 0, n_q = 1;
+  bool nodes = false;  // the lowest energies may go through the frequency-node or moment kernel
   int64_t n_chunks = 1, n_items = 0;
   double *part = nullptr;
   size_t part_cap = 0;  // doubles
@@ -129,6 +130,10 @@ int configure(rad_plan p, const Choice &c) {
   p->n_q = 1;
   p->n_chunks = 1;
   const bool per_particle = (p->want & RAD_PER_PARTICLE) != 0;
+  // the node and moment forms go with the default launch shape; a caller that sets another asks for
+  // that direct kernel
+  const Choice def = default_choice(p->precision, p->mode, p->n_omega);
+  const bool def_shape = c.R == def.R && c.NW == def.NW && c.T == def.T && c.pp == def.pp;
   if (per_particle) {
     p->n_chunks = std::max<int64_t>(p->n_particles, 1);  // one chunk per particle: partials are per particle
   } else if (tiles > 0 && tiles < target) {
@@ -165,6 +170,7 @@ int configure(rad_plan p, const Choice &c) {
   sh.grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(p->n_items, resident)));
   p->shape = sh;
   p->choice = c;
+  p->nodes = p->precision == RAD_MIXED && c.pp && def_shape && node_path_allowed(sh, p->n_omega, p->n_angles, p->n_chunks);
   const size_t need = static_cast<size_t>(std::max<int64_t>(per_chunk * p->n_chunks, 1));
   if (need > p->part_cap) {
     if (p->part) cudaFree(p->part);
@@ -234,11 +240,13 @@ Params make_params(rad_plan p, const double *samples, const int64_t *offsets, co
   P.counter = p->ctrl;
   P.status = p->ctrl + 1;
   P.table = table;
-  // control block: [0] work counter, [1] status, bytes 16..47 the grid maxima of RAD_MIXED's guard
+  // control block: [0] work counter, [1] status, [2] node cut, [3] node kernel's work counter, bytes 16..47 the grid maxima of RAD_MIXED's guard
   P.phase_budget = p->phase_budget;
   P.grid_max = p->precision == RAD_MIXED
                    ? reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(p->ctrl) + 16)
                    : nullptr;
+  P.node_cut = p->nodes ? p->ctrl + 2 : nullptr;
+  P.counter2 = p->ctrl + 3;
   return P;
 }
 
@@ -287,14 +295,18 @@ int execute(rad_plan p, const double *samples, const int64_t *offsets, const dou
   Params P = make_params(p, samples, offsets, gamma, energy, weight, hw, tx, ty, table);
   e = cudaMemsetAsync(p->ctrl, 0, kCtrlBytes, st);
   if (e != cudaSuccess) return cuda_fail(e);
-  e = launch_validate(P, d_omega, need_dom, bin_of_angle, st);
+  NodeCost nc;
+  if (p->nodes && p->precision == RAD_MIXED) {
+    nc = node_cost(p->n_omega, p->shape.R);
+  }
+  e = launch_validate(P, d_omega, need_dom, bin_of_angle, nc, st);
   if (e != cudaSuccess) return cuda_fail(e);
   LaunchShape sh = p->shape;
   if (p->precision == RAD_MIXED && p->choice.pp) {
     e = launch_prep_samples(P, sh.T, p->prep, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
-  if (p->timing) {  // events bracket the integral kernel alone
+  if (p->timing) {  // events bracket the integral kernels alone
     e = cudaEventRecord(p->ev0, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
@@ -303,6 +315,10 @@ int execute(rad_plan p, const double *samples, const int64_t *offsets, const dou
   } else if (p->precision == RAD_FP64_DF) {
     e = launch_df(P, &sh, st);
   } else if (p->choice.pp) {
+    if (p->nodes) {
+      e = launch_mixed_nodes(P, p->prep, p->sms, st);
+      if (e != cudaSuccess) return cuda_fail(e);
+    }
     e = launch_mixed_pp(P, p->prep, &sh, st);
   } else {
     e = launch_mixed(P, &sh, st);
@@ -372,7 +388,8 @@ int plan_create(int64_t ns, int64_t np, int64_t no, int64_t na, int mode, int pr
     cudaFree(p->ctrl);
     cudaFree(p->cube_new);
     if (p->part) cudaFree(p->part);
-    delete p;
+    if (p->prep) cudaFree(p->prep);
+      delete p;
     return rc;
   }
   *out = p;
@@ -525,7 +542,8 @@ int rad_plan_last_kernel_ms(rad_plan plan, double *ms) {
 int rad_plan_kernel_launches(rad_plan plan) {
   if (!plan) return 0;
   if (plan->n_omega == 0 || plan->n_angles == 0) return 0;
-  const int pre = (plan->precision == RAD_MIXED && plan->choice.pp) ? 1 : 0;  // pre-pass
+  // pre-pass; node or moment kernel
+  const int pre = (plan->precision == RAD_MIXED && plan->choice.pp ? 1 : 0) + (plan->nodes ? 1 : 0);
   if (plan->want & RAD_PER_PARTICLE) return 3 + pre;  // validate, main, per-particle reduce
   int n = 3 + pre;  // validate, main, finalize
   if (plan->want & 6) n += 1;

@@ -69,6 +69,11 @@ struct Params {
   // of non-negative doubles (zeroed before launch): [0] max |theta_x|, [1] max |theta_y|,
   // [2] max (theta_x^2 + theta_y^2)/2, [3] max hw (eV). They bound the in-tile phase offsets.
   unsigned long long *grid_max;
+  // number of lowest energies that k_mixed_nodes (RAD_MIXED) sums instead of
+  // the direct kernel, chosen on the device (null: none), and that kernel's work counter (zeroed before
+  // launch)
+  int *node_cut;
+  int *counter2;
   double phase_budget;  // RAD_MIXED: largest accepted in-tile phase-offset bound (radians)
 };
 
@@ -250,6 +255,18 @@ bool shape_supported_mixed_pp(int R, int NW, int T);
 int occupancy_mixed_pp(const LaunchShape &s, int mode = RAD_SPIN_HALF);
 cudaError_t launch_prep_samples(const Params &P, int T, float *prep, cudaStream_t st);
 cudaError_t launch_mixed_pp(const Params &P, const float *prep, LaunchShape *shape, cudaStream_t st);
+// frequency-node kernel for the lowest energies of the pre-pass form (rad_mixed_nodes.cu)
+bool node_path_allowed(const LaunchShape &s, int64_t n_omega, int64_t n_angles, int64_t n_chunks);
+// Chooses on the device how many of the lowest energies the node (or moment) kernel takes. Costs per
+// sample and direction in SM clocks: `direct` per energy summed directly; `fixed` per tile of `tile`
+// energies and `per_energy` per energy over the run length, which is the number of samples within a
+// phase range of `reach` radians over the tile's span of w*, at most `cap`.
+struct NodeCost {
+  int gran = 64, tile = 512, from_zero = 1;
+  float direct = 0.f, fixed = 0.f, per_energy = 0.f, reach = 0.f, cap = 64.f;
+};
+NodeCost node_cost(int64_t n_omega, int direct_r);
+cudaError_t launch_mixed_nodes(const Params &P, const float *prep, int sms, cudaStream_t st);
 
 // FP64-accurate kernel with double-float FP32 arithmetic after the FP64 phase (rad_df.cu)
 bool shape_supported_df(int R, int NW, int T);
@@ -258,7 +275,7 @@ cudaError_t launch_df(const Params &P, LaunchShape *shape, cudaStream_t st);
 
 // post-processing kernels (rad_post.cu)
 cudaError_t launch_validate(const Params &P, const double *d_omega, bool need_domega,
-                            const int32_t *bin_of_angle, cudaStream_t st);
+                            const int32_t *bin_of_angle, const NodeCost &cost, cudaStream_t st);
 cudaError_t launch_finalize(const Params &P, double *cube_new, double *out_cube, int accumulate,
                             cudaStream_t st);
 // k_finalize (S-mode partials) publishing a failed call status into *publish_status.

@@ -44,4 +44,28 @@ __device__ __forceinline__ void tile_base_sincos(float wt_hi, float wt_lo, float
   __sincosf(rr * kTwoPiF, &s0, &c0);
 }
 
+// Turns of the product beyond 2^21, in FP64; out of line so that the compiler does not speculate its
+// FP64 instructions (16 SM clocks each) into the common path.
+__device__ __noinline__ inline float far_turns(float wt_hi, float wt_lo, float a0h, float a0l) {
+  const double ph = (static_cast<double>(wt_hi) + static_cast<double>(wt_lo)) *
+                    (static_cast<double>(a0h) + static_cast<double>(a0l));
+  return static_cast<float>(ph - rint(ph));
+}
+
+// The same without w*/2pi in FP64: beyond 2^21 turns it is formed from the pair.
+__device__ __forceinline__ void tile_base_sincos(float wt_hi, float wt_lo, float a0h, float a0l, float &s0, float &c0) {
+  const float p = wt_hi * a0h;
+  float e = fmaf(wt_hi, a0h, -p);
+  e = fmaf(wt_hi, a0l, e);
+  e = fmaf(wt_lo, a0h, e);
+  float rr;
+  if (fabsf(p) < 2097152.0f) {
+    const float nr = __fsub_rn(__fadd_rn(p, kMagicF), kMagicF);
+    rr = __fadd_rn(__fsub_rn(p, nr), e);
+  } else {
+    rr = far_turns(wt_hi, wt_lo, a0h, a0l);
+  }
+  __sincosf(rr * kTwoPiF, &s0, &c0);
+}
+
 }  // namespace rad

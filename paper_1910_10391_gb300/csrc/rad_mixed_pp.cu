@@ -174,7 +174,12 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? (R <= 2 ? 2 : 1) : 3) k_mix
   __syncthreads();
   uint32_t full_par[2] = {0u, 0u};   // consumers: next parity of full[s]
   uint32_t uses[2] = {0u, 0u};       // producer (thread 0): copies issued into stage s so far
-  const int64_t per_chunk = static_cast<int64_t>(P.n_wt) * P.n_nt;
+  // energies below node_cut (a multiple of 32 R, or all of them) are summed by k_mixed_nodes
+  const int64_t cut = P.node_cut ? *P.node_cut : 0;
+  const int wt0 = static_cast<int>((cut + 32 * R - 1) / (32 * R)), n_wt = P.n_wt - wt0;
+  const int64_t per_chunk = static_cast<int64_t>(n_wt) * P.n_nt;
+  const int64_t n_items = per_chunk * P.n_chunks;
+  if (n_wt <= 0) return;
   int s = 0;
 
   // thread 0: wait until every warp released stage st's previous tile, then fill it
@@ -195,10 +200,10 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? (R <= 2 ? 2 : 1) : 3) k_mix
     __syncthreads();
     const int64_t item = s_item[0];
     __syncthreads();
-    if (item >= P.n_items) break;
+    if (item >= n_items) break;
     const int64_t chunk = item / per_chunk;
     const int64_t rem = item % per_chunk;
-    const int nt = static_cast<int>(rem / P.n_wt), wt = static_cast<int>(rem % P.n_wt);
+    const int nt = static_cast<int>(rem / n_wt), wt = wt0 + static_cast<int>(rem % n_wt);
     const int64_t jdir = static_cast<int64_t>(nt) * NW + warp;
     const bool jvalid = jdir < P.n_angles;
     const double nx = jvalid ? P.theta_x[jdir] : 0.0;

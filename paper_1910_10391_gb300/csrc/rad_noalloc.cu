@@ -122,7 +122,7 @@ extern "C" int rad_spectrum_noalloc(const double *samples, int64_t n_samples_tot
 
   // the work counter and status words must start at zero on every call
   e = cudaMemsetAsync(ctrl, 0, kCtrlBytes, st);
-  if (e == cudaSuccess) e = launch_validate(P, nullptr, false, nullptr, st);
+  if (e == cudaSuccess) e = launch_validate(P, nullptr, false, nullptr, NodeCost{}, st);
   if (e == cudaSuccess) e = launch_mixed(P, &sh, st);
   // combine: the cube is written once (cube_new and the output are the same array)
   if (e == cudaSuccess) e = launch_finalize_status(P, out_cube, out_cube, 0, ctrl + 2, st);

@@ -14,11 +14,77 @@ namespace {
 
 __device__ __forceinline__ bool finite_d(double v) { return isfinite(v); }
 
+// Chooses how many of the lowest energies go through the node or moment kernel (0: none), from the
+// trajectories' mean phase length per sample and the costs in c_ (see NodeCost). One block of 256
+// threads; the energies must ascend (else none). It runs beside the checks, so it trusts no input:
+// offsets outside the records count for nothing, and other bad values only move a cut that the
+// failed check keeps from being used.
+__device__ void node_plan(const Params &P, const NodeCost &c_) {
+  __shared__ double s_dA[256], s_n[256];
+  const int tid = threadIdx.x;
+  bool bad = false;
+  for (int64_t i = tid; i + 1 < P.n_omega; i += 256) bad |= !(P.hw[i] <= P.hw[i + 1]);
+  // up to 16 particles x 16 directions spread over the call
+  double dA = 0.0, cnt = 0.0;
+  if (P.n_particles > 0) {
+    const int64_t p = (tid >> 4) * P.n_particles / 16;
+    const int64_t j = ((tid & 15) * P.n_angles + P.n_angles / 2) / 16;
+    const int64_t ka = P.offsets[p], kb = P.offsets[p + 1];
+    if (ka >= 0 && kb - ka >= 2 && kb <= P.n_samples_total) {
+      const double *a = P.samples + ka * kRec, *b = P.samples + (kb - 1) * kRec;
+      const double nx = P.theta_x[j], ny = P.theta_y[j], g = P.gamma[p];
+      const double c = 1.0 / (2.0 * g * g) + (nx * nx + ny * ny) * 0.5;
+      dA = fabs(c * (b[F_T] - a[F_T]) - (b[F_DZ] - a[F_DZ]) - nx * (b[F_X] - a[F_X]) - ny * (b[F_Y] - a[F_Y]));
+      cnt = static_cast<double>(kb - ka - 1);
+    }
+  }
+  s_dA[tid] = dA;
+  s_n[tid] = cnt;
+  bad = __syncthreads_or(bad);
+  for (int o = 128; o > 0; o >>= 1) {
+    if (tid < o) {
+      s_dA[tid] += s_dA[tid + o];
+      s_n[tid] += s_n[tid + o];
+    }
+    __syncthreads();
+  }
+  if (tid != 0 || bad || P.n_particles == 0) return;
+  const double step = s_dA[0] / s_n[0];
+  const double E = P.energy[0];
+  auto ws = [&](int64_t i) {
+    const double h = P.hw[i], w = h / kHbarC;
+    return P.mode == RAD_CLASSICAL ? w : w / (1.0 - h / E);
+  };
+  const int64_t gran = c_.gran, tile = c_.tile;
+  float best = c_.direct * static_cast<float>(P.n_omega), done = 0.f;  // done: whole tiles below
+  int64_t cut = 0;
+  double lo = 0.0;
+  for (int64_t e = 0; e < P.n_omega; e += gran) {
+    const int64_t t0 = e / tile * tile;
+    const int64_t end = e + gran < P.n_omega ? e + gran : P.n_omega;
+    if (e == t0) lo = c_.from_zero ? 0.0 : ws(t0);
+    const double span = (ws(end - 1) - lo) * step;
+    const float runlen = fminf(fmaxf(static_cast<float>(c_.reach / fmax(span, 1e-30)), 1.f), c_.cap);
+    const float part = c_.fixed + c_.per_energy * static_cast<float>(end - t0) / runlen;
+    const float total = done + part + c_.direct * static_cast<float>(P.n_omega - end);
+    if (total < best) {
+      best = total;
+      cut = end;
+    }
+    if (end == t0 + tile) done += part;
+  }
+  *P.node_cut = static_cast<int>(cut);
+}
+
 // One grid-stride pass over every device input; any violation sets RAD_EDATA.
-__global__ void k_validate(const Params P, const double *d_omega, int need_domega,
-                           double max_hw_unused) {
-  (void)max_hw_unused;
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+// With a node cut to choose, the grid has one more block, which does that.
+__global__ void k_validate(const Params P, const double *d_omega, int need_domega, const NodeCost cost) {
+  const int n_blocks = static_cast<int>(gridDim.x) - (P.node_cut ? 1 : 0);
+  if (static_cast<int>(blockIdx.x) == n_blocks) {
+    node_plan(P, cost);
+    return;
+  }
+  const int64_t stride = static_cast<int64_t>(n_blocks) * blockDim.x;
   const int64_t t0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   bool bad = false;
   // particles
@@ -324,7 +390,7 @@ int *device_status_word(cudaError_t *err) {
 }
 
 cudaError_t launch_validate(const Params &P, const double *d_omega, bool need_domega,
-                            const int32_t *bin_of_angle, cudaStream_t st) {
+                            const int32_t *bin_of_angle, const NodeCost &cost, cudaStream_t st) {
   (void)bin_of_angle;
   int sms = 0, dev = 0;
   cudaGetDevice(&dev);
@@ -334,7 +400,7 @@ cudaError_t launch_validate(const Params &P, const double *d_omega, bool need_do
   const int64_t cap = static_cast<int64_t>(sms > 0 ? sms : 1) * 8;
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
-  k_validate<<<static_cast<int>(blocks), 256, 0, st>>>(P, d_omega, need_domega ? 1 : 0, 0.0);
+  k_validate<<<static_cast<int>(blocks) + (P.node_cut ? 1 : 0), 256, 0, st>>>(P, d_omega, need_domega ? 1 : 0, cost);
   return cudaGetLastError();
 }
 
