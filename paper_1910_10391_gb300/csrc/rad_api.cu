@@ -50,6 +50,9 @@ struct rad_plan_s {
   LaunchShape shape{};
   int n_wt = 0, n_nt = 0, amp_mode = 0, n_q = 1;
   bool nodes = false;  // the lowest energies may go through the frequency-node or moment kernel
+  int cheb_grid = 0;   // resident blocks of the moment kernel (FP64 forms)
+  unsigned char *cheb_scratch = nullptr;
+  size_t cheb_cap = 0;
   int64_t n_chunks = 1, n_items = 0;
   double *part = nullptr;
   size_t part_cap = 0;  // doubles
@@ -105,6 +108,12 @@ bool same_choice(const Choice &a, const Choice &b) {
   return a.R == b.R && a.NW == b.NW && a.T == b.T && a.chunk_mult == b.chunk_mult && a.pp == b.pp && a.pe == b.pe;
 }
 
+// Fewest energies for which the FP64 forms consider the moment kernel: its fixed cost per sample is
+// that of 7 energies summed by k_fp64, or 25 by k_df (cheb_cost).
+constexpr int64_t kChebMinFp64 = 24, kChebMinDf = 64;
+// Partials that a finer split for the moment kernel may take (doubles).
+constexpr int64_t kChebPartials = int64_t(1) << 26;
+
 // Work decomposition for a choice; (re)allocates scratch when it grows.
 int configure(rad_plan p, const Choice &c) {
   if (!supported(p->precision, c)) return RAD_EINVAL;
@@ -134,6 +143,13 @@ int configure(rad_plan p, const Choice &c) {
   // that direct kernel
   const Choice def = default_choice(p->precision, p->mode, p->n_omega);
   const bool def_shape = c.R == def.R && c.NW == def.NW && c.T == def.T && c.pp == def.pp;
+  const bool df = p->precision == RAD_FP64_DF;
+  bool cheb = p->precision != RAD_MIXED && def_shape && p->n_omega >= (df ? kChebMinDf : kChebMinFp64) &&
+              p->n_omega <= INT32_MAX && p->n_angles >= 16 && p->n_particles > 0;
+  const int cheb_occ = cheb ? occupancy_cheb(p->mode, df) : 0;
+  cheb = cheb_occ > 0;
+  const int64_t cheb_res = static_cast<int64_t>(p->sms) * cheb_occ;
+  const int64_t ctiles = cheb ? cheb_tiles(p->mode, p->n_omega, p->n_angles) : 1;
   if (per_particle) {
     p->n_chunks = std::max<int64_t>(p->n_particles, 1);  // one chunk per particle: partials are per particle
   } else if (tiles > 0 && tiles < target) {
@@ -150,6 +166,37 @@ int configure(rad_plan p, const Choice &c) {
     }
   }
   const int ncomp = ncomp_of(p->mode);
+  if (cheb && !per_particle && p->n_chunks * ctiles < 2 * cheb_res) {
+    // the moment kernel has an eighth or less of the direct kernel's work items per chunk: split finer
+    const int64_t bins = std::max<int64_t>(p->n_omega * p->n_angles, 1);
+    if (!p->amp_mode && p->n_particles * ctiles >= 2 * cheb_res) {
+      p->n_chunks = std::min<int64_t>(p->n_particles, std::max<int64_t>(p->n_chunks, kChebPartials / bins));
+    } else {
+      // time pieces of at least 2 tiles; of the counts, the one whose last wave is fullest
+      const int64_t avg_len = p->n_samples_total / p->n_particles;
+      const int64_t most = std::min<int64_t>({std::max<int64_t>(avg_len / (2 * c.T), 1),
+                                              (4 * cheb_res + ctiles * p->n_particles - 1) / (ctiles * p->n_particles),
+                                              std::max<int64_t>(kChebPartials / (bins * ncomp * p->n_particles), 1)});
+      const int64_t least = p->amp_mode ? std::min<int64_t>(p->n_q, most) : 1;
+      double best = 1e300;
+      int64_t nq = least;
+      for (int64_t v = least; v <= most; ++v) {
+        const int64_t waves = (v * p->n_particles * ctiles + cheb_res - 1) / cheb_res;
+        const double t = static_cast<double>(waves) / static_cast<double>(v) * (1.0 + 0.01 * static_cast<double>(waves));
+        if (t < best) {
+          best = t;
+          nq = v;
+        }
+      }
+      if (nq > 1 || p->amp_mode) {
+        p->amp_mode = 1;
+        p->n_q = static_cast<int>(nq);
+        p->n_chunks = p->n_particles * nq;
+      } else {
+        p->n_chunks = std::max<int64_t>(p->n_chunks, std::min<int64_t>(p->n_particles, kChebPartials / bins));
+      }
+    }
+  }
   // keep the partials within 4 GiB
   const int64_t per_chunk = p->n_omega * p->n_angles * (p->amp_mode ? ncomp : 1);
   const int64_t cap_chunks = per_chunk > 0 ? std::max<int64_t>(1, (int64_t(1) << 29) / per_chunk) : 1;
@@ -170,7 +217,24 @@ int configure(rad_plan p, const Choice &c) {
   sh.grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(p->n_items, resident)));
   p->shape = sh;
   p->choice = c;
-  p->nodes = p->precision == RAD_MIXED && c.pp && def_shape && node_path_allowed(sh, p->n_omega, p->n_angles, p->n_chunks);
+  p->nodes = p->precision == RAD_MIXED ? c.pp && def_shape && node_path_allowed(sh, p->n_omega, p->n_angles, p->n_chunks)
+                                       : cheb && ctiles <= (INT32_MAX - 65536) / p->n_chunks;
+  if (p->precision != RAD_MIXED && p->nodes) {
+    p->cheb_grid = static_cast<int>(std::min<int64_t>(ctiles * p->n_chunks, cheb_res));
+    const size_t bytes = cheb_scratch_bytes(p->mode, p->cheb_grid);
+    if (bytes > p->cheb_cap) {
+      if (p->cheb_scratch) cudaFree(p->cheb_scratch);
+      p->cheb_scratch = nullptr;
+      p->cheb_cap = 0;
+      cudaError_t e = cudaMalloc(&p->cheb_scratch, bytes);
+      if (e != cudaSuccess) {  // no room: the direct kernel alone
+        (void)cudaGetLastError();
+        p->nodes = false;
+      } else {
+        p->cheb_cap = bytes;
+      }
+    }
+  }
   const size_t need = static_cast<size_t>(std::max<int64_t>(per_chunk * p->n_chunks, 1));
   if (need > p->part_cap) {
     if (p->part) cudaFree(p->part);
@@ -298,6 +362,13 @@ int execute(rad_plan p, const double *samples, const int64_t *offsets, const dou
   NodeCost nc;
   if (p->nodes && p->precision == RAD_MIXED) {
     nc = node_cost(p->n_omega, p->shape.R);
+  } else if (p->nodes) {
+    const bool df = p->precision == RAD_FP64_DF;
+    nc = cheb_cost(p->mode, df, 32 * p->shape.R * (df ? p->shape.NW : 1));
+    // idle lanes of the last direction tile cost as much as the others
+    const float waste = static_cast<float>((p->n_angles + 31) / 32 * 32) / static_cast<float>(p->n_angles);
+    nc.fixed *= waste;
+    nc.per_energy *= waste;
   }
   e = launch_validate(P, d_omega, need_dom, bin_of_angle, nc, st);
   if (e != cudaSuccess) return cuda_fail(e);
@@ -308,6 +379,11 @@ int execute(rad_plan p, const double *samples, const int64_t *offsets, const dou
   }
   if (p->timing) {  // events bracket the integral kernels alone
     e = cudaEventRecord(p->ev0, st);
+    if (e != cudaSuccess) return cuda_fail(e);
+  }
+  if (p->precision != RAD_MIXED && p->nodes) {
+    const bool df = p->precision == RAD_FP64_DF;
+    e = launch_cheb(P, df, p->cheb_scratch, p->cheb_grid, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
   if (p->precision == RAD_FP64) {
@@ -389,7 +465,8 @@ int plan_create(int64_t ns, int64_t np, int64_t no, int64_t na, int mode, int pr
     cudaFree(p->cube_new);
     if (p->part) cudaFree(p->part);
     if (p->prep) cudaFree(p->prep);
-      delete p;
+    if (p->cheb_scratch) cudaFree(p->cheb_scratch);
+    delete p;
     return rc;
   }
   *out = p;
@@ -403,6 +480,7 @@ void plan_free(rad_plan p) {
   if (p->ev0) cudaEventDestroy(p->ev0);
   if (p->ev1) cudaEventDestroy(p->ev1);
   if (p->part) cudaFree(p->part);
+  if (p->cheb_scratch) cudaFree(p->cheb_scratch);
   if (p->cube_new) cudaFree(p->cube_new);
   if (p->ctrl) cudaFree(p->ctrl);
   delete p;

@@ -1,0 +1,596 @@
+// FP64 and FP64-accurate radiation integral through Chebyshev moments (sm_103a).
+//
+// The direct kernels (rad_fp64.cu, rad_df.cu) evaluate one sin/cos per (sample, photon energy,
+// direction). Over a run of samples whose phase lengths a_k from the run's centre stay within
+// a_lim, the factor e^{i w a_k} of every photon energy w <= w_hi is a short Chebyshev series in
+// x_k = a_k / a_lim (Jacobi-Anger):
+//   e^{i w a_k} = sum_m (2 - delta_m0) i^m J_m(w a_lim) T_m(x_k),
+// so the run's amplitude is a combination of kM real moments that do not depend on the energy:
+//   sum_k f_k e^{i w a_k} = sum_m (2 - delta_m0) i^m J_m(w a_lim) M_m,  M_m = sum_k f_k T_m(x_k).
+// A sample then costs one recurrence step and one multiply-add per component and moment whatever
+// the number of energies, and an energy costs kM multiply-adds per component, one sin/cos of the
+// run's base phase and one rotation per run instead of per sample. With w_hi a_lim = 9 (5 for
+// spin 1/2, which has three components and keeps 24 moments instead of 32) the first dropped term is
+// below 1e-14; terms that are below 1e-18 at an energy's own w a_lim are left out for it.
+//
+// Work split: a block of 4 warps takes 32 directions (one per lane: x_k, the recurrence and the
+// moments live in the lane's registers and need no exchange) and the energies of one tile. The warps
+// take a quarter of a run's samples each, add their moments through shared memory and then take a
+// quarter of the energies each. Amplitudes are kept in a block's own scratch, [energy][component]
+// [lane], one coalesced read and write per run and energy.
+//
+// DF = false: everything FP64. DF = true: the phase lengths, f and the base phase are formed in
+// FP64, the moments, the series and the rotations in the float-pair arithmetic of rad_df.cu
+// (products by FMA, Ogita-Rump-Oishi Dot2 sums), because GB300 executes FP64 at 1/64 of its FP32
+// rate: a float-pair multiply-add takes about a sixth of the time of an FP64 one.
+#include <type_traits>
+
+#include "rad_df_reduce.cuh"
+#include "rad_fp64_sincos.cuh"
+#include "rad_internal.cuh"
+
+namespace rad {
+namespace {
+
+constexpr int kW = 4;        // warps per block
+constexpr int kWin = 256;    // samples of a window, the longest run
+constexpr int kRecW = 10;    // doubles per prepared sample
+
+template <int MODE>
+struct Cheb {
+  static constexpr bool kSpin = MODE == RAD_SPIN_HALF;
+  static constexpr int NP = kSpin ? 3 : 2;   // summed components (f_x, f_y, j)
+  static constexpr int kM = kSpin ? 24 : 32;
+  static constexpr double kPhi = kSpin ? 5.0 : 9.0;
+  static constexpr int kTile = kSpin ? 256 : 512;  // energies of a tile
+};
+
+// float pair
+struct df2 {
+  float h, l;
+};
+
+__device__ __forceinline__ df2 df_norm(float a, float b) {  // |a| >= |b|
+  const float s = __fadd_rn(a, b);
+  return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+
+// 2 x t - u
+__device__ __forceinline__ df2 df_rec(const df2 &x2, const df2 &t, const df2 &u) {
+  const float p = __fmul_rn(x2.h, t.h);
+  float e = __fmaf_rn(x2.h, t.h, -p);
+  e = __fmaf_rn(x2.h, t.l, __fmaf_rn(x2.l, t.h, e));
+  float s, r;
+  dfr::two_sum(p, -u.h, s, r);
+  return df_norm(s, __fadd_rn(r, __fsub_rn(e, u.l)));
+}
+
+__device__ __forceinline__ df2 to_df(double v) {
+  df2 r;
+  dfr::split_df(v, r.h, r.l);
+  return r;
+}
+
+__device__ __forceinline__ void async16(void *dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
+// running sum of products and its value as a number of the arithmetic
+template <bool DF>
+struct Num;
+template <>
+struct Num<false> {
+  using T = double;
+  using A = double;
+  static __device__ __forceinline__ A zero() { return 0.0; }
+  static __device__ __forceinline__ T from(double v) { return v; }
+  static __device__ __forceinline__ T rec(T x2, T t, T u) { return fma(x2, t, -u); }
+  static __device__ __forceinline__ T neg(T v) { return -v; }
+  static __device__ __forceinline__ void mac(A &a, T x, T y) { a = fma(x, y, a); }
+  static __device__ __forceinline__ void add(A &a, T x) { a += x; }
+  static __device__ __forceinline__ T value(A a) { return a; }
+  static __device__ __forceinline__ double to_double(A a) { return a; }
+};
+template <>
+struct Num<true> {
+  using T = df2;
+  using A = df2;  // h: leading sum, l: sum of the errors (not normalised)
+  static __device__ __forceinline__ A zero() { return {0.f, 0.f}; }
+  static __device__ __forceinline__ T from(double v) { return to_df(v); }
+  static __device__ __forceinline__ T rec(const T &x2, const T &t, const T &u) { return df_rec(x2, t, u); }
+  static __device__ __forceinline__ T neg(const T &v) { return {-v.h, -v.l}; }
+  static __device__ __forceinline__ void mac(A &a, const T &x, const T &y) { dfr::dot2(a.h, a.l, x.h, x.l, y.h, y.l); }
+  static __device__ __forceinline__ void add(A &a, const T &x) {
+    float s, t;
+    dfr::two_sum(a.h, x.h, s, t);
+    a.h = s;
+    a.l = __fadd_rn(a.l, __fadd_rn(t, x.l));
+  }
+  static __device__ __forceinline__ T value(const A &a) {
+    float s, t;
+    dfr::two_sum(a.h, a.l, s, t);
+    return {s, t};
+  }
+  static __device__ __forceinline__ double to_double(const A &a) {
+    return static_cast<double>(a.h) + static_cast<double>(a.l);
+  }
+};
+
+// A block's scratch: amplitudes [tile][2 NP][32], particle sums S [tile][32], series coefficients
+// [tile][kM], w* [tile], number of terms [tile], and (DF) the float-pair sin/cos table.
+template <int MODE>
+struct Scratch {
+  using C = Cheb<MODE>;
+  static constexpr size_t kAmp = 0;
+  static constexpr size_t kS = kAmp + size_t(C::kTile) * 2 * C::NP * 32 * 8;
+  static constexpr size_t kCoef = kS + size_t(C::kTile) * 32 * 8;
+  static constexpr size_t kWs = kCoef + size_t(C::kTile) * C::kM * 8;
+  static constexpr size_t kTerms = kWs + size_t(C::kTile) * 8;
+  static constexpr size_t kTab = kTerms + size_t(C::kTile) * 4;
+  static constexpr size_t kTotal = kTab + dfr::kTabN * 16;
+};
+
+template <int MODE>
+struct Smem {
+  using C = Cheb<MODE>;
+  static constexpr int kRecs = 0;                                    // double [256][10]
+  static constexpr int kMom = kRecs + kWin * kRecW * 8;              // 8 bytes [4][NP kM][32]
+  static constexpr int kStep = kMom + kW * C::NP * C::kM * 32 * 8;   // float4 [256]
+  // per warp, two slots: series coefficients and amplitudes of the energy at hand and of the next one
+  static constexpr int kSlot = C::kM * 8 + 2 * C::NP * 32 * 8;
+  static constexpr int kRing = kStep + kWin * 16;
+  static constexpr int kMisc = kRing + kW * 2 * kSlot;               // item, status; float [4]
+  static constexpr int kTotal = kMisc + 64;
+};
+
+// (2 - delta_m0) (-1)^{m/2} J_m(z) for m < M into out (as T), and the number of terms above 1e-18,
+// rounded up to even. Power series below z = 1/2, Miller's backward recurrence normalised by
+// J_0 + 2 sum J_2k = 1 above (M. Abramowitz, I. A. Stegun, 9.12).
+template <bool DF, int M>
+__device__ int bessel_row(double z, typename Num<DF>::T *out) {
+  int terms = 2;
+  auto put = [&](int m, double j) {
+    const double v = (m ? 2.0 : 1.0) * ((m >> 1) & 1 ? -j : j);
+    out[m] = Num<DF>::from(v);
+    if (fabs(v) > 1e-18 && m + 1 > terms) terms = m + 1;
+  };
+  if (z < 0.5) {
+    const double q = -0.25 * z * z;
+    double lead = 1.0;  // (z/2)^m / m!
+    for (int m = 0; m < M; ++m) {
+      double s = 1.0, t = 1.0;
+      for (int k = 1; k < 9; ++k) {
+        t *= q / (k * static_cast<double>(m + k));
+        s += t;
+      }
+      put(m, lead * s);
+      lead *= 0.5 * z / (m + 1);
+    }
+  } else {
+    const double rz = 2.0 / z;
+    // twice: the normalising sum first, then the values (no array of them)
+    double hi = 0.0, lo = 1e-200, sum = 0.0;
+    for (int m = 60; m > 0; --m) {
+      const double t = fma(m * rz, lo, -hi);  // J_{m-1}
+      hi = lo;
+      lo = t;
+      if ((m - 1) % 2 == 0) sum += (m - 1 ? 2.0 : 1.0) * t;
+    }
+    const double scale = 1.0 / sum;
+    hi = 0.0;
+    lo = 1e-200;
+    for (int m = 60; m > 0; --m) {
+      const double t = fma(m * rz, lo, -hi);
+      hi = lo;
+      lo = t;
+      if (m - 1 < M) put(m - 1, t * scale);
+    }
+  }
+  return (terms + 1) & ~1;
+}
+
+template <int MODE, bool DF>
+__global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned char *__restrict__ scratch_all) {
+  using C = Cheb<MODE>;
+  using N = Num<DF>;
+  using T = typename N::T;
+  using A = typename N::A;
+  using SM = Smem<MODE>;
+  using SC = Scratch<MODE>;
+  constexpr int NP = C::NP, kM = C::kM, kTile = C::kTile;
+  constexpr int NC = C::kSpin ? 8 : 6;
+  static_assert(sizeof(T) == 8 && sizeof(A) == 8, "8-byte numbers");
+  extern __shared__ __align__(128) unsigned char sm[];
+  double *recs = reinterpret_cast<double *>(sm + SM::kRecs);
+  A *s_mom = reinterpret_cast<A *>(sm + SM::kMom);
+  float4 *s_step = reinterpret_cast<float4 *>(sm + SM::kStep);
+  int *s_item = reinterpret_cast<int *>(sm + SM::kMisc);
+  float *s_max = reinterpret_cast<float *>(s_item + 2);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+
+  if (tid == 0) s_item[1] = *reinterpret_cast<volatile int *>(P.status);
+  __syncthreads();
+  if (s_item[1] != 0) return;
+  const int64_t cut = *P.node_cut;  // energies [0, cut) are summed here, the others by the direct kernel
+  if (cut <= 0) return;
+  unsigned char *scr = scratch_all + static_cast<size_t>(blockIdx.x) * SC::kTotal;
+  A *amp = reinterpret_cast<A *>(scr + SC::kAmp);
+  double *Ssum = reinterpret_cast<double *>(scr + SC::kS);
+  T *coef = reinterpret_cast<T *>(scr + SC::kCoef);
+  double *wsv = reinterpret_cast<double *>(scr + SC::kWs);
+  int *n_terms = reinterpret_cast<int *>(scr + SC::kTerms);
+  float4 *tab = reinterpret_cast<float4 *>(scr + SC::kTab);
+  if (DF)
+    for (int i = tid; i < dfr::kTabN; i += kW * 32) tab[i] = dfr::table_pair(P.table[2 * i]);
+
+  const int64_t n_wt = (cut + kTile - 1) / kTile, n_dt = (P.n_angles + 31) / 32;
+  const int64_t per_chunk = n_wt * n_dt, n_items = per_chunk * P.n_chunks;
+  int64_t have_wt = -1;
+  double have_E = -1.0, a_lim = 0.0;
+
+  for (;;) {
+    __syncthreads();
+    if (tid == 0) s_item[0] = atomicAdd(P.counter2, 1);
+    __syncthreads();
+    const int64_t item = s_item[0];
+    if (item >= n_items) break;
+    const int64_t chunk = item / per_chunk, rem = item % per_chunk;
+    const int64_t dt = rem / n_wt, wt = rem % n_wt;
+    const int64_t jdir = dt * 32 + lane;
+    const int64_t jread = jdir < P.n_angles ? jdir : P.n_angles - 1;
+    const double nx = P.theta_x[jread], ny = P.theta_y[jread];
+    const double th2h = (nx * nx + ny * ny) * 0.5;
+    const int64_t e0 = wt * kTile;
+    const int ne = static_cast<int>(cut - e0 < kTile ? cut - e0 : kTile);
+    int64_t p0, p1;
+    int q;
+    chunk_range(P, chunk, p0, p1, q);
+    // component c (I_x, I_y, I_z, J as re, im) of an energy from its summed ones
+    auto comp = [&](const double *a, int c) {
+      if (c < 4) return a[c];
+      if (c < 6) return -fma(nx, a[c - 4], ny * a[c - 2]);
+      return a[c - 2];
+    };
+    for (int64_t p = p0; p < p1; ++p) {
+      const int64_t off = P.offsets[p], len = P.offsets[p + 1] - off;
+      const int64_t kb = P.amp_mode ? (len * q) / P.n_q : 0, ke = P.amp_mode ? (len * (q + 1)) / P.n_q : len;
+      const double *S = P.samples + off * kRec;
+      const double gam = P.gamma[p], En = P.energy[p];
+      const double inv2g2 = 1.0 / (2.0 * gam * gam), cn = inv2g2 + th2h;
+      if (wt != have_wt || (MODE != RAD_CLASSICAL && En != have_E)) {  // series of the tile's energies
+        have_wt = wt;
+        have_E = En;
+        auto ws_of = [&](double h) {
+          const double w = __ddiv_rn(h, kHbarC);
+          return MODE == RAD_CLASSICAL ? w : __ddiv_rn(w, __dsub_rn(1.0, __ddiv_rn(h, En)));
+        };
+        a_lim = C::kPhi / ws_of(P.hw[e0 + ne - 1]);  // the energies ascend
+        __syncthreads();  // the last particle's series is no longer read
+        for (int e = tid; e < ne; e += kW * 32) {
+          const double w = ws_of(P.hw[e0 + e]);
+          wsv[e] = w;
+          n_terms[e] = bessel_row<DF, kM>(w * a_lim, coef + static_cast<size_t>(e) * kM);
+        }
+        __syncthreads();
+      }
+      const double inv_a = 1.0 / a_lim;
+      const double cns = cn * inv_a, nxs = nx * inv_a, nys = ny * inv_a;
+      const float cnf = static_cast<float>(cn), nxf = static_cast<float>(nx), nyf = static_cast<float>(ny);
+      bool first = true;  // first run of the particle's piece: amplitudes are written, not added to
+      for (int64_t w0 = kb; w0 < ke; w0 += kWin) {
+        const int n = static_cast<int>(ke - w0 < kWin ? ke - w0 : kWin);
+        const double *r0 = S + w0 * kRec;  // the window's reference
+        __syncthreads();  // the last window's records are no longer read
+        for (int k = tid; k < n; k += kW * 32) {
+          const double *rc = r0 + k * kRec;
+          const int64_t K = w0 + k;
+          const double tm = K == 0 ? rc[F_T] : rc[F_T - kRec], tp = K == len - 1 ? rc[F_T] : rc[F_T + kRec];
+          const double w = 0.5 * (tp - tm);
+          double *o = recs + k * kRecW;
+          o[0] = rc[F_T] - r0[F_T];
+          o[1] = rc[F_DZ] - r0[F_DZ];
+          o[2] = rc[F_X] - r0[F_X];
+          o[3] = rc[F_Y] - r0[F_Y];
+          o[4] = rc[F_VX];
+          o[5] = rc[F_VY];
+          o[6] = rc[F_AX] * w;
+          o[7] = rc[F_AY] * w;
+          o[8] = rc[F_AZ] * w;
+          o[9] = rc[F_DVZ];
+          // step to the next sample (none after the window's last)
+          const double *rn = k + 1 < n ? rc + kRec : rc;
+          s_step[k] = make_float4(static_cast<float>(rn[F_T] - rc[F_T]), static_cast<float>(rn[F_DZ] - rc[F_DZ]),
+                                static_cast<float>(rn[F_X] - rc[F_X]), static_cast<float>(rn[F_Y] - rc[F_Y]));
+        }
+        __syncthreads();
+        // widest step in phase length over the window and the block's directions, FP32 with a margin
+        // for its rounding; runs of L samples span at most (L - 1) of it
+        float st = 0.f;
+        for (int k = warp; k < n; k += kW) {
+          const float4 d = s_step[k];
+          const float a = cnf * d.x, b = nxf * d.z, c = nyf * d.w;
+          const float v = fabsf(a - d.y - b - c) + 4e-7f * (fabsf(a) + fabsf(d.y) + fabsf(b) + fabsf(c));
+          st = v > st || v != v ? v : st;  // a NaN stays
+          if (st != st) break;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const float v = __shfl_xor_sync(0xffffffffu, st, o);
+          st = v > st || v != v ? v : st;
+        }
+        if (lane == 0) s_max[warp] = st;
+        __syncthreads();
+        int run = kWin;
+        {
+          float m = s_max[0];
+#pragma unroll
+          for (int i = 1; i < kW; ++i) m = s_max[i] > m || s_max[i] != s_max[i] ? s_max[i] : m;
+          const float lim = static_cast<float>(2.0 * a_lim);
+          // the fewest runs of about equal length; a NaN step gives runs of one sample
+          const float most = m > 0.f ? fminf(lim / m, static_cast<float>(kWin)) + 1.f : m == 0.f ? kWin : 1.f;
+          run = most < 2.f ? 1 : static_cast<int>(most);
+          run = run > kWin ? kWin : run;
+          const int runs = (n + run - 1) / run;
+          run = (n + runs - 1) / runs;
+        }
+        const double A0 = ((cn * r0[F_T] - r0[F_DZ]) - nx * r0[F_X]) - ny * r0[F_Y];
+        for (int k0 = 0; k0 < n; k0 += run) {
+          const int m = n - k0 < run ? n - k0 : run;  // samples of this run
+          auto length = [&](int k) {  // phase length from the window's reference
+            const double *o = recs + k * kRecW;
+            return fma(-ny, o[3], fma(-nx, o[2], fma(cn, o[0], -o[1])));
+          };
+          const double ctr = 0.5 * (length(k0) + length(k0 + m - 1));
+          const double off_x = -ctr * inv_a;
+          A M[kM][NP];
+#pragma unroll
+          for (int i = 0; i < kM; ++i)
+#pragma unroll
+            for (int c = 0; c < NP; ++c) M[i][c] = N::zero();
+          const int share = (m + kW - 1) / kW;
+          const int ka = k0 + min(warp * share, m), kz = k0 + min((warp + 1) * share, m);
+          for (int k = ka; k < kz; ++k) {
+            const double *o = recs + k * kRecW;
+            const double x = fma(-nys, o[3], fma(-nxs, o[2], fma(-inv_a, o[1], fma(cns, o[0], off_x))));
+            const double vx = o[4], vy = o[5];
+            const double D = cn - o[9] - nx * vx - ny * vy;  // 1 - n.beta (Sec. II, g)
+            // 1 / D by one cubic step from the hardware's 20-bit reciprocal
+            double r;
+            asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(D));
+            const double eps = fma(-D, r, 1.0);
+            r = fma(fma(eps, eps, eps), r, r);
+            const double g = r * r;
+            const double a = nx - vx, b = ny - vy;
+            const double mm = fma(ny, o[7], fma(nx, o[6], o[8]));  // n.beta_dot, weighted
+            T f[NP];
+            f[0] = N::from(fma(a, mm, -o[6] * D) * g);
+            f[1] = N::from(fma(b, mm, -o[7] * D) * g);
+            if (C::kSpin) f[NP - 1] = N::from(mm * g);
+            // T_{m+2} = 2 T_2 T_m - T_{m-2}: the even and the odd orders as two chains of half the
+            // length, which quarters the growth of the recurrence's rounding near x = +-1
+            const T x1 = N::from(x), t2x2 = N::from(fma(4.0 * x, x, -2.0));
+            T ev0 = N::from(1.0), od0 = x1;          // T_0, T_1
+            T ev1 = N::from(fma(2.0 * x, x, -1.0));  // T_2
+            T od1 = N::rec(t2x2, x1, x1);            // T_3 = 2 T_2 T_1 - T_1
+#pragma unroll
+            for (int i = 0; i < kM; i += 2) {
+#pragma unroll
+              for (int c = 0; c < NP; ++c) {
+                if (i == 0)
+                  N::add(M[0][c], f[c]);
+                else
+                  N::mac(M[i][c], f[c], ev0);
+                N::mac(M[i + 1][c], f[c], od0);
+              }
+              if (i + 4 < kM) {
+                const T e2 = N::rec(t2x2, ev1, ev0), o2 = N::rec(t2x2, od1, od0);
+                ev0 = ev1;
+                ev1 = e2;
+                od0 = od1;
+                od1 = o2;
+              } else {
+                ev0 = ev1;
+                od0 = od1;
+              }
+            }
+          }
+          // moments of the run: the warps' shares, added in a fixed order, a quarter of them per warp
+          __syncthreads();  // the last run's moments are no longer read
+#pragma unroll
+          for (int i = 0; i < kM; ++i)
+#pragma unroll
+            for (int c = 0; c < NP; ++c) s_mom[((warp * kM + i) * NP + c) * 32 + lane] = M[i][c];
+          __syncthreads();
+          for (int i = warp; i < kM * NP; i += kW) {
+            A v = s_mom[i * 32 + lane];
+#pragma unroll
+            for (int w = 1; w < kW; ++w) N::add(v, N::value(s_mom[(w * kM * NP + i) * 32 + lane]));
+            reinterpret_cast<T *>(s_mom)[i * 32 + lane] = N::value(v);
+          }
+          __syncthreads();
+          T Mv[kM][NP];
+#pragma unroll
+          for (int i = 0; i < kM; ++i)
+#pragma unroll
+            for (int c = 0; c < NP; ++c) Mv[i][c] = reinterpret_cast<const T *>(s_mom)[(i * NP + c) * 32 + lane];
+          const double Ac = A0 + ctr;
+          // the next energy's coefficients and amplitudes are on their way from L2 while this one's
+          // series is summed: eight warps an SM are too few to hide those loads
+          unsigned char *ring = sm + SM::kRing + warp * 2 * SM::kSlot;
+          auto fetch = [&](int e, int slot) {
+            if (e < ne) {
+              unsigned char *d = ring + slot * SM::kSlot;
+              const unsigned char *c = reinterpret_cast<const unsigned char *>(coef + static_cast<size_t>(e) * kM);
+              if (lane < kM / 2) async16(d + lane * 16, c + lane * 16);
+              if (!first) {
+                const unsigned char *a = reinterpret_cast<const unsigned char *>(amp + static_cast<size_t>(e) * 2 * NP * 32);
+#pragma unroll
+                for (int i = 0; i < NP; ++i) async16(d + kM * 8 + (i * 32 + lane) * 16, a + (i * 32 + lane) * 16);
+              }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+          };
+          fetch(warp, 0);
+          int slot = 0;
+          for (int e = warp; e < ne; e += kW, slot ^= 1) {
+            fetch(e + kW, slot ^ 1);
+            const int terms = n_terms[e];
+            const double phi = __dmul_rn(wsv[e], Ac);
+            T sn, cs;
+            float4 entry;
+            float xh, xl;
+            if constexpr (DF) entry = tab[dfr::reduce_phase(phi, xh, xl) & (dfr::kTabN - 1)];
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            __syncwarp();
+            const T *cf = reinterpret_cast<const T *>(ring + slot * SM::kSlot);
+            const A *old = reinterpret_cast<const A *>(ring + slot * SM::kSlot + kM * 8) + lane;
+            A re[NP], im[NP];
+#pragma unroll
+            for (int c = 0; c < NP; ++c) re[c] = im[c] = N::zero();
+#pragma unroll
+            for (int i = 0; i < kM; i += 2) {
+              if (i < terms) {
+                const T ce = cf[i], co = cf[i + 1];
+#pragma unroll
+                for (int c = 0; c < NP; ++c) {
+                  N::mac(re[c], ce, Mv[i][c]);
+                  N::mac(im[c], co, Mv[i + 1][c]);
+                }
+              }
+            }
+            if constexpr (DF)
+              dfr::sincos_from_entry(entry, xh, xl, sn.h, sn.l, cs.h, cs.l);
+            else
+              sincos_table(phi, P.table, sn, cs);
+            A *o = amp + static_cast<size_t>(e) * 2 * NP * 32 + lane;
+#pragma unroll
+            for (int c = 0; c < NP; ++c) {
+              A zr = first ? N::zero() : old[(2 * c) * 32], zi = first ? N::zero() : old[(2 * c + 1) * 32];
+              const T vr = N::value(re[c]), vi = N::value(im[c]);
+              N::mac(zr, cs, vr);
+              N::mac(zr, N::neg(sn), vi);
+              N::mac(zi, sn, vr);
+              N::mac(zi, cs, vi);
+              o[(2 * c) * 32] = zr;
+              o[(2 * c + 1) * 32] = zi;
+            }
+            __syncwarp();  // the slot is read; the fetch after next refills it
+          }
+          first = false;
+        }
+      }
+      // the particle's (piece's) amplitudes: each warp its own energies
+      for (int e = warp; e < ne; e += kW) {
+        double a[2 * NP];
+#pragma unroll
+        for (int c = 0; c < 2 * NP; ++c)
+          a[c] = first ? 0.0 : N::to_double(amp[(static_cast<size_t>(e) * 2 * NP + c) * 32 + lane]);
+        if (P.amp_mode) {
+          if (jdir < P.n_angles) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) P.part[((chunk * NC + c) * P.n_angles + jdir) * P.n_omega + e0 + e] = comp(a, c);
+          }
+          continue;
+        }
+        double I2 = 0.0;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+          const double v = comp(a, c);
+          I2 = fma(v, v, I2);
+        }
+        double Sv = I2;
+        if (MODE != RAD_CLASSICAL) {
+          const double u = P.hw[e0 + e] / En;
+          if (MODE == RAD_SPIN0) {
+            Sv = (1.0 - u) * I2;
+          } else {
+            const double J2 = a[2 * NP - 2] * a[2 * NP - 2] + a[2 * NP - 1] * a[2 * NP - 1];
+            Sv = 0.5 * (1.0 + (1.0 - u) * (1.0 - u)) * I2 + (u * u) / (2.0 * gam * gam) * J2;
+          }
+        }
+        const double wp = P.weight ? P.weight[p] : 1.0;
+        const double acc = fma(wp, Sv, p == p0 ? 0.0 : Ssum[e * 32 + lane]);
+        if (p + 1 < p1)
+          Ssum[e * 32 + lane] = acc;
+        else if (jdir < P.n_angles)
+          P.part[(chunk * P.n_angles + jdir) * P.n_omega + e0 + e] = acc;
+      }
+    }
+    if (p0 >= p1 && !P.amp_mode && jdir < P.n_angles)  // no particles: an empty sum
+      for (int e = warp; e < ne; e += kW) P.part[(chunk * P.n_angles + jdir) * P.n_omega + e0 + e] = 0.0;
+  }
+}
+
+template <int MODE, bool DF>
+cudaError_t occ_t(int *nb) {
+  auto kern = k_cheb<MODE, DF>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<MODE>::kTotal);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, kern, kW * 32, Smem<MODE>::kTotal);
+}
+
+template <int MODE, bool DF>
+cudaError_t launch_t(const Params &P, unsigned char *scratch, int grid, cudaStream_t st) {
+  auto kern = k_cheb<MODE, DF>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<MODE>::kTotal);
+  if (e != cudaSuccess) return e;
+  kern<<<grid, kW * 32, Smem<MODE>::kTotal, st>>>(P, scratch);
+  return cudaGetLastError();
+}
+
+template <typename F>
+cudaError_t by_mode(int mode, F f) {
+  switch (mode) {
+    case RAD_CLASSICAL: return f(std::integral_constant<int, RAD_CLASSICAL>{});
+    case RAD_SPIN0: return f(std::integral_constant<int, RAD_SPIN0>{});
+    case RAD_SPIN_HALF: return f(std::integral_constant<int, RAD_SPIN_HALF>{});
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+}  // namespace
+
+int64_t cheb_tiles(int mode, int64_t n_omega, int64_t n_angles) {
+  const int64_t tile = cheb_tile(mode);
+  return (n_omega + tile - 1) / tile * ((n_angles + 31) / 32);
+}
+
+int cheb_tile(int mode) { return mode == RAD_SPIN_HALF ? Cheb<RAD_SPIN_HALF>::kTile : Cheb<RAD_CLASSICAL>::kTile; }
+
+int occupancy_cheb(int mode, bool df) {
+  int nb = 0;
+  const cudaError_t e = by_mode(mode, [&](auto m) {
+    return df ? occ_t<decltype(m)::value, true>(&nb) : occ_t<decltype(m)::value, false>(&nb);
+  });
+  return e == cudaSuccess ? nb : 0;
+}
+
+size_t cheb_scratch_bytes(int mode, int grid) {
+  return static_cast<size_t>(grid) *
+         (mode == RAD_SPIN_HALF ? Scratch<RAD_SPIN_HALF>::kTotal : Scratch<RAD_CLASSICAL>::kTotal);
+}
+
+// Cost per sample and direction in SM clocks, for the choice of the cut (measured rates of the
+// kernels): per energy summed directly; per sample for the moments; per energy and run for the
+// series; reach: the phase range of a run.
+NodeCost cheb_cost(int mode, bool df, int direct_gran) {
+  NodeCost c;
+  const bool spin = mode == RAD_SPIN_HALF;
+  c.gran = direct_gran;
+  c.tile = cheb_tile(mode);
+  c.cap = kWin;
+  c.reach = 0.8f * 2.f * static_cast<float>(spin ? Cheb<RAD_SPIN_HALF>::kPhi : Cheb<RAD_CLASSICAL>::kPhi);
+  c.direct = df ? (spin ? 1.25f : 1.05f) : (spin ? 10.2f : 9.2f);
+  c.fixed = df ? 26.f : 60.f;
+  c.per_energy = df ? 6.f : (spin ? 40.f : 35.f);
+  return c;
+}
+
+cudaError_t launch_cheb(const Params &P, bool df, unsigned char *scratch, int grid, cudaStream_t st) {
+  return by_mode(P.mode, [&](auto m) {
+    return df ? launch_t<decltype(m)::value, true>(P, scratch, grid, st)
+              : launch_t<decltype(m)::value, false>(P, scratch, grid, st);
+  });
+}
+
+}  // namespace rad

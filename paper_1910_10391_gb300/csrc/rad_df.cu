@@ -35,33 +35,8 @@
 namespace rad {
 namespace {
 
-constexpr int kDfTabN = 2048;  // table of (cos, sin)(2 pi j / 2048): every other FP64 table entry
-using dfr::reduce_phase;
-using dfr::split_df;
-
-// s + t = a + b exactly (Knuth)
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &t) {
-  s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  t = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-
-// s + t = a + b exactly when |a| >= |b| or a = 0 (Dekker)
-__device__ __forceinline__ void fast_two_sum(float a, float b, float &s, float &t) {
-  s = __fadd_rn(a, b);
-  t = __fsub_rn(b, __fsub_rn(s, a));
-}
-
-// one Dot2 step: (S, C) += (fh + fl)(eh + el)
-__device__ __forceinline__ void dot2(float &S, float &C, float fh, float fl, float eh, float el) {
-  const float p = __fmul_rn(fh, eh);
-  float q = __fmaf_rn(fh, eh, -p);                 // exact error of the product
-  q = __fmaf_rn(fh, el, __fmaf_rn(fl, eh, q));     // cross terms
-  float s, t;
-  two_sum(S, p, s, t);
-  S = s;
-  C = __fadd_rn(C, __fadd_rn(t, q));
-}
+constexpr int kDfTabN = dfr::kTabN;
+using dfr::dot2;
 
 template <int MODE>
 struct DfNcomp {
@@ -121,10 +96,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 5 : 2) k_df(const Params P)
   // (cos, sin)(2 pi j / 2048) as float pairs (c_hi, c_lo, s_hi, s_lo) from every other entry of the
   // FP64 table (2048 entries, 32 KB)
   for (int i = tid; i < kDfTabN; i += NW * 32) {
-    const double2 t = P.table[2 * i];
-    const float ch = __double2float_rn(t.x), sh = __double2float_rn(t.y);
-    tab[i] = make_float4(ch, __double2float_rn(t.x - static_cast<double>(ch)), sh,
-                         __double2float_rn(t.y - static_cast<double>(sh)));
+    tab[i] = dfr::table_pair(P.table[2 * i]);
   }
   if (tid == 0) {
     mbar_init(&bar[0], 1);
@@ -137,7 +109,12 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 5 : 2) k_df(const Params P)
   float4 *sFa = reinterpret_cast<float4 *>(sm + L::kNk + T * 8);   // (fx_hi, fx_lo, fy_hi, fy_lo)
   float2 *sFj = reinterpret_cast<float2 *>(sm + L::kNk + T * 24);  // (j_hi, j_lo), spin 1/2 only
 
-  const int64_t per_chunk = static_cast<int64_t>(P.n_wt) * P.n_nt;
+  // energies below node_cut (a multiple of NW 32 R, or all of them) are summed by k_cheb
+  const int64_t cut = P.node_cut ? *P.node_cut : 0;
+  const int wt0 = static_cast<int>((cut + NW * 32 * R - 1) / (NW * 32 * R)), n_wt = P.n_wt - wt0;
+  if (n_wt <= 0) return;
+  const int64_t per_chunk = static_cast<int64_t>(n_wt) * P.n_nt;
+  const int64_t n_items = per_chunk * P.n_chunks;
   int s = 0;
 
   for (;;) {
@@ -145,13 +122,13 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 5 : 2) k_df(const Params P)
     __syncthreads();
     const int64_t item = s_item[0];
     __syncthreads();
-    if (item >= P.n_items) break;
+    if (item >= n_items) break;
     const int64_t chunk = item / per_chunk;
     const int64_t rem = item % per_chunk;
     // one direction per item, shared by the block's warps (the per-sample preparation is done
     // once for all of them); warp w takes the energies (wt NW + w) 32 R + 32 r + lane
-    const int64_t jdir = rem / P.n_wt;
-    const int wt = static_cast<int>(rem % P.n_wt);
+    const int64_t jdir = rem / n_wt;
+    const int wt = wt0 + static_cast<int>(rem % n_wt);
     const double nx = P.theta_x[jdir];
     const double ny = P.theta_y[jdir];
     const double th2h = __dmul_rn(__dadd_rn(__dmul_rn(nx, nx), __dmul_rn(ny, ny)), 0.5);
@@ -266,34 +243,8 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 5 : 2) k_df(const Params P)
 #pragma unroll
           for (int r = 0; r < R; ++r) {
             const double phi = __dmul_rn(ws[r], A);
-            float xh, xl;
-            const int j = reduce_phase(phi, xh, xl);
-            const float4 t = tab[j & (kDfTabN - 1)];  // (C_hi, C_lo, S_hi, S_lo)
-            const float x2 = __fmul_rn(xh, xh);
-            const float x2e = __fmaf_rn(xh, xh, -x2);  // xh^2 = x2 + x2e exactly
-            // cos x - 1 and the part of sin x below xh
-            const float cm = __fmaf_rn(-0.5f, x2e, __fmaf_rn(-xh, xl, __fmul_rn(x2, __fmaf_rn(x2, 1.0f / 24.0f, -0.5f))));
-            const float sxl = __fmaf_rn(__fmul_rn(-xh, x2), __fmaf_rn(x2, -1.0f / 120.0f, 1.0f / 6.0f), xl);
-            // sin(phi) = S + S cm + C xh + C sxl. The table's leading parts are 0 at multiples of pi/2
-            // (filled by exact symmetry) and at least sin(2 pi/2048) = 3.07e-3 in magnitude elsewhere,
-            // twice |C xh| <= pi/2048, so Fast2Sum gives the exact sum of S and C xh
-            float sh, sl;
-            {
-              const float p = __fmul_rn(t.x, xh);
-              const float pe = __fmaf_rn(t.x, xh, -p);
-              float v;
-              fast_two_sum(t.z, p, sh, v);
-              sl = __fadd_rn(v, __fadd_rn(pe, __fmaf_rn(t.y, xh, __fmaf_rn(t.x, sxl, __fmaf_rn(t.z, cm, t.w)))));
-            }
-            // cos(phi) = C + C cm - S xh - S sxl
-            float ch, cl;
-            {
-              const float p = __fmul_rn(-t.z, xh);
-              const float pe = __fmaf_rn(-t.z, xh, -p);
-              float v;
-              fast_two_sum(t.x, p, ch, v);
-              cl = __fadd_rn(v, __fadd_rn(pe, __fmaf_rn(-t.w, xh, __fmaf_rn(-t.z, sxl, __fmaf_rn(t.x, cm, t.y)))));
-            }
+            float sh, sl, ch, cl;
+            dfr::sincos_df(phi, tab, sh, sl, ch, cl);
             dot2(tS[r][0], tC[r][0], Fa.x, Fa.y, ch, cl);
             dot2(tS[r][1], tC[r][1], Fa.x, Fa.y, sh, sl);
             dot2(tS[r][2], tC[r][2], Fa.z, Fa.w, ch, cl);

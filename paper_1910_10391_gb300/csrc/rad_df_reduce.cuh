@@ -119,5 +119,73 @@ __device__ __forceinline__ int reduce_phase(double phi, float &xh, float &xl) {
   return j;
 }
 
+// s + t = a + b exactly (Knuth)
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &t) {
+  s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  t = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+
+// s + t = a + b exactly when |a| >= |b| or a = 0 (Dekker)
+__device__ __forceinline__ void fast_two_sum(float a, float b, float &s, float &t) {
+  s = __fadd_rn(a, b);
+  t = __fsub_rn(b, __fsub_rn(s, a));
+}
+
+// one Dot2 step: (S, C) += (fh + fl)(eh + el)
+__device__ __forceinline__ void dot2(float &S, float &C, float fh, float fl, float eh, float el) {
+  const float p = __fmul_rn(fh, eh);
+  float q = __fmaf_rn(fh, eh, -p);                 // exact error of the product
+  q = __fmaf_rn(fh, el, __fmaf_rn(fl, eh, q));     // cross terms
+  float s, t;
+  two_sum(S, p, s, t);
+  S = s;
+  C = __fadd_rn(C, __fadd_rn(t, q));
+}
+
+constexpr int kTabN = 2048;  // table of (cos, sin)(2 pi j / 2048): every other FP64 table entry
+
+// (cos, sin) of a table entry as float pairs (c_hi, c_lo, s_hi, s_lo)
+__device__ __forceinline__ float4 table_pair(double2 t) {
+  const float ch = __double2float_rn(t.x), sh = __double2float_rn(t.y);
+  return make_float4(ch, __double2float_rn(t.x - static_cast<double>(ch)), sh,
+                     __double2float_rn(t.y - static_cast<double>(sh)));
+}
+
+// sin(phi) = sh + sl, cos(phi) = ch + cl from the phase's table entry t = (C_hi, C_lo, S_hi, S_lo) and
+// Taylor series of its remainder (xh, xl)
+__device__ __forceinline__ void sincos_from_entry(const float4 &t, float xh, float xl, float &sh, float &sl, float &ch,
+                                                  float &cl) {
+  const float x2 = __fmul_rn(xh, xh);
+  const float x2e = __fmaf_rn(xh, xh, -x2);  // xh^2 = x2 + x2e exactly
+  // cos x - 1 and the part of sin x below xh
+  const float cm = __fmaf_rn(-0.5f, x2e, __fmaf_rn(-xh, xl, __fmul_rn(x2, __fmaf_rn(x2, 1.0f / 24.0f, -0.5f))));
+  const float sxl = __fmaf_rn(__fmul_rn(-xh, x2), __fmaf_rn(x2, -1.0f / 120.0f, 1.0f / 6.0f), xl);
+  // sin(phi) = S + S cm + C xh + C sxl. The table's leading parts are 0 at multiples of pi/2
+  // (filled by exact symmetry) and at least sin(2 pi/2048) = 3.07e-3 in magnitude elsewhere,
+  // twice |C xh| <= pi/2048, so Fast2Sum gives the exact sum of S and C xh
+  {
+    const float p = __fmul_rn(t.x, xh);
+    const float pe = __fmaf_rn(t.x, xh, -p);
+    float v;
+    fast_two_sum(t.z, p, sh, v);
+    sl = __fadd_rn(v, __fadd_rn(pe, __fmaf_rn(t.y, xh, __fmaf_rn(t.x, sxl, __fmaf_rn(t.z, cm, t.w)))));
+  }
+  // cos(phi) = C + C cm - S xh - S sxl
+  {
+    const float p = __fmul_rn(-t.z, xh);
+    const float pe = __fmaf_rn(-t.z, xh, -p);
+    float v;
+    fast_two_sum(t.x, p, ch, v);
+    cl = __fadd_rn(v, __fadd_rn(pe, __fmaf_rn(-t.w, xh, __fmaf_rn(-t.z, sxl, __fmaf_rn(t.x, cm, t.y)))));
+  }
+}
+
+__device__ __forceinline__ void sincos_df(double phi, const float4 *tab, float &sh, float &sl, float &ch, float &cl) {
+  float xh, xl;
+  const int j = reduce_phase(phi, xh, xl);
+  sincos_from_entry(tab[j & (kTabN - 1)], xh, xl, sh, sl, ch, cl);
+}
+
 }  // namespace dfr
 }  // namespace rad

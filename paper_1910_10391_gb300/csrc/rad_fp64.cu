@@ -16,34 +16,10 @@
 // being summed.
 #include <cstdio>
 
-#include "rad_internal.cuh"
+#include "rad_fp64_sincos.cuh"
 
 namespace rad {
 namespace {
-
-// 2 pi / kTabN = pi * 2^-11 split into the double nearest pi and its remainder, both
-// scaled by 2^-11 (exact): C1 + C2 = 2 pi / 4096 to about 106 bits.
-constexpr double kPiHi = 3.141592653589793116;        // nearest double to pi
-constexpr double kPiLo = 1.2246467991473531772e-16;   // pi - kPiHi (rounded)
-constexpr double kC1 = kPiHi / 2048.0;
-constexpr double kC2 = kPiLo / 2048.0;
-constexpr double kInvStep = 2048.0 / 3.141592653589793238462643383279502884;  // 4096/(2 pi)
-constexpr double kMagic = 6755399441055744.0;  // 1.5 * 2^52: adding it rounds to an integer
-
-__device__ __forceinline__ void sincos_table(double phi, const double2 *__restrict__ tab, double &s,
-                                             double &c) {
-  const double y = fma(phi, kInvStep, kMagic);  // round(phi * 4096/(2 pi)) + magic
-  const int j = __double2loint(y);              // low word holds the integer (two's complement)
-  const double jd = y - kMagic;                 // exact
-  double r = fma(-jd, kC1, phi);
-  r = fma(-jd, kC2, r);
-  const double2 t = tab[j & (kTabN - 1)];       // (cos, sin)(2 pi j / 4096)
-  const double r2 = r * r;
-  const double sr = fma(r2 * r, -1.0 / 6.0, r);           // sin r
-  const double cm = r2 * fma(r2, 1.0 / 24.0, -0.5);       // cos r - 1
-  s = fma(t.x, sr, fma(t.y, cm, t.y));                    // sin(a + r)
-  c = fma(-t.y, sr, fma(t.x, cm, t.x));                   // cos(a + r)
-}
 
 template <int MODE>
 struct Ncomp {
@@ -102,7 +78,12 @@ __global__ void __launch_bounds__(NW * 32) k_fp64(const Params P) {
   double *myFx = myA + T, *myFy = myA + 2 * T;
   double *myJ = myA + 3 * T;  // spin-1/2 only
 
-  const int64_t per_chunk = static_cast<int64_t>(P.n_wt) * P.n_nt;
+  // energies below node_cut (a multiple of 32 R, or all of them) are summed by k_cheb
+  const int64_t cut = P.node_cut ? *P.node_cut : 0;
+  const int wt0 = static_cast<int>((cut + 32 * R - 1) / (32 * R)), n_wt = P.n_wt - wt0;
+  if (n_wt <= 0) return;
+  const int64_t per_chunk = static_cast<int64_t>(n_wt) * P.n_nt;
+  const int64_t n_items = per_chunk * P.n_chunks;
   int s = 0;  // stage of the next tile to consume
 
   for (;;) {
@@ -110,10 +91,10 @@ __global__ void __launch_bounds__(NW * 32) k_fp64(const Params P) {
     __syncthreads();
     const int64_t item = s_item[0];
     __syncthreads();
-    if (item >= P.n_items) break;
+    if (item >= n_items) break;
     const int64_t chunk = item / per_chunk;
     const int64_t rem = item % per_chunk;
-    const int nt = static_cast<int>(rem / P.n_wt), wt = static_cast<int>(rem % P.n_wt);
+    const int nt = static_cast<int>(rem / n_wt), wt = wt0 + static_cast<int>(rem % n_wt);
     const int64_t jdir = static_cast<int64_t>(nt) * NW + warp;
     const bool jvalid = jdir < P.n_angles;
     const double nx = jvalid ? P.theta_x[jdir] : 0.0;

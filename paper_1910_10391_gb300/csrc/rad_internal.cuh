@@ -69,7 +69,7 @@ struct Params {
   // of non-negative doubles (zeroed before launch): [0] max |theta_x|, [1] max |theta_y|,
   // [2] max (theta_x^2 + theta_y^2)/2, [3] max hw (eV). They bound the in-tile phase offsets.
   unsigned long long *grid_max;
-  // number of lowest energies that k_mixed_nodes (RAD_MIXED) sums instead of
+  // number of lowest energies that k_mixed_nodes (RAD_MIXED) or k_cheb (the FP64 forms) sums instead of
   // the direct kernel, chosen on the device (null: none), and that kernel's work counter (zeroed before
   // launch)
   int *node_cut;
@@ -272,6 +272,14 @@ cudaError_t launch_mixed_nodes(const Params &P, const float *prep, int sms, cuda
 bool shape_supported_df(int R, int NW, int T);
 int occupancy_df(const LaunchShape &s, int mode = RAD_SPIN_HALF);
 cudaError_t launch_df(const Params &P, LaunchShape *shape, cudaStream_t st);
+
+// Chebyshev-moment kernel of the FP64 forms for the lowest energies (rad_cheb.cu)
+int64_t cheb_tiles(int mode, int64_t n_omega, int64_t n_angles);  // work items per chunk
+int cheb_tile(int mode);                                          // energies per tile
+int occupancy_cheb(int mode, bool df);
+size_t cheb_scratch_bytes(int mode, int grid);
+NodeCost cheb_cost(int mode, bool df, int direct_gran);
+cudaError_t launch_cheb(const Params &P, bool df, unsigned char *scratch, int grid, cudaStream_t st);
 
 // post-processing kernels (rad_post.cu)
 cudaError_t launch_validate(const Params &P, const double *d_omega, bool need_domega,
