@@ -1,5 +1,5 @@
 """Planar trajectories from the tabulated potential (k_channel_tab): particle counts around the block
-grid and the switch from four lanes to one lane per particle, positions far outside the first cell and
+grid and the switch from eight lanes to one lane per particle, positions far outside the first cell and
 on cell borders and uneven lengths,
 against the trajectory oracle. Tolerance as for the FP64 records elsewhere: 1e-9 of a field's scale
 (the table's first dropped term is below 1e-16 of the narrowest Gaussian)."""
@@ -49,3 +49,19 @@ def test_neighbour_counts(K):
     lengths = np.full(6, 400)
     got, _, off = run_gpu(channel(-1, ALL), lib, x0, th, E, lengths, dt, 2)
     check(got, off, range(6), x0, th, lengths, E, dt, 2, -1, ALL, orc)
+
+
+@pytest.mark.parametrize("n", [608, 609])
+def test_axial_warp_and_half_warp(n):
+    """Axial particles on both sides of the switch from a warp to 16 lanes each."""
+    import test_axial_gpu as X
+    lib, orc = X.potentials(K=1)
+    E, dt = 10e9, 5e-9
+    x0, y0, thx, thy = X.entries(n, E, orc.lat, seed=6)
+    lengths = 20 + np.arange(n) % 5
+    got, _, off = X.run_gpu(X.channel(-1, ALL), lib, x0, y0, thx, thy, E, lengths, dt, 4)
+    for p in (0, 1, n // 2, n - 1):
+        ref = T.axial_trajectories(x0[p:p + 1], y0[p:p + 1], thx[p:p + 1], thy[p:p + 1], E, int(lengths[p]), dt, 4, orc,
+                                   charge=-1, ms=True, ms_el=True, ll=True, ms_loss=True,
+                                   particle_ids=np.array([p], dtype=np.int64))
+        X.close(got[off[p]:off[p + 1]], ref[0])
