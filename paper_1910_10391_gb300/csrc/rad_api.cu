@@ -88,11 +88,12 @@ ShapeKey key_of(int dev, int64_t ns, int64_t np, int64_t no, int64_t na, int mod
 // Defaults before any autotuning: the fastest shapes on the 10 GeV positron ensemble (512 hw x
 // 64 x 64 directions, 32 particles per launch). The mixed kernel runs 8 warps per block, 2 blocks
 // per SM; spin-1/2 keeps every sin/cos on the SFU, classical and spin-0 (two fewer sums per term)
-// take 1/8 of them on the FMA pipe. k_df's blocks of 4 warps take 256 energies of one direction
-// (128 when the grid has no more).
-Choice default_choice(int precision, int mode, int64_t n_omega) {
+// take 1/8 of them on the FMA pipe. k_df's blocks of 4 warps take 128 energies of one
+// direction: the moment kernel takes the lowest ones in steps of as many, and 256 per block (3 % fewer
+// instructions per term) left half of a block idle for the 128 highest of 384.
+Choice default_choice(int precision, int mode) {
   if (precision == RAD_FP64) return Choice{2, 8, 64, 1, 0};
-  if (precision == RAD_FP64_DF) return Choice{n_omega <= 128 ? 1 : 2, 4, 64, 1, 0};
+  if (precision == RAD_FP64_DF) return Choice{1, 4, 64, 1, 0};
   if (mode == RAD_SPIN_HALF) return Choice{2, 8, 256, 1, 1, 0};
   return Choice{2, 8, 256, 1, 1, 6};
 }
@@ -141,7 +142,7 @@ int configure(rad_plan p, const Choice &c) {
   const bool per_particle = (p->want & RAD_PER_PARTICLE) != 0;
   // the node and moment forms go with the default launch shape; a caller that sets another asks for
   // that direct kernel
-  const Choice def = default_choice(p->precision, p->mode, p->n_omega);
+  const Choice def = default_choice(p->precision, p->mode);
   const bool def_shape = c.R == def.R && c.NW == def.NW && c.T == def.T && c.pp == def.pp;
   const bool df = p->precision == RAD_FP64_DF;
   bool cheb = p->precision != RAD_MIXED && def_shape && p->n_omega >= (df ? kChebMinDf : kChebMinFp64) &&
@@ -172,17 +173,23 @@ int configure(rad_plan p, const Choice &c) {
     if (!p->amp_mode && p->n_particles * ctiles >= 2 * cheb_res) {
       p->n_chunks = std::min<int64_t>(p->n_particles, std::max<int64_t>(p->n_chunks, kChebPartials / bins));
     } else {
-      // time pieces of at least 2 tiles; of the counts, the one whose last wave is fullest
+      // time pieces of at least 2 tiles; of the counts, the one with the least time by the kernel's costs (cheb_cost)
       const int64_t avg_len = p->n_samples_total / p->n_particles;
       const int64_t most = std::min<int64_t>({std::max<int64_t>(avg_len / (2 * c.T), 1),
                                               (4 * cheb_res + ctiles * p->n_particles - 1) / (ctiles * p->n_particles),
                                               std::max<int64_t>(kChebPartials / (bins * ncomp * p->n_particles), 1)});
       const int64_t least = p->amp_mode ? std::min<int64_t>(p->n_q, most) : 1;
+      // FP64: one block's four warps fill an SM's FP64 pipe, so an SM is one slot; float pairs need the
+      // latency hiding of all resident blocks
+      const int64_t slots = df ? cheb_res : p->sms;
+      const NodeCost nc = cheb_cost(p->mode, df, 0);
       double best = 1e300;
       int64_t nq = least;
       for (int64_t v = least; v <= most; ++v) {
-        const int64_t waves = (v * p->n_particles * ctiles + cheb_res - 1) / cheb_res;
-        const double t = static_cast<double>(waves) / static_cast<double>(v) * (1.0 + 0.01 * static_cast<double>(waves));
+        const int64_t waves = (v * p->n_particles * ctiles + slots - 1) / slots, piece = (avg_len + v - 1) / v;
+        const double series = static_cast<double>(std::min<int64_t>(p->n_omega, nc.tile)) * nc.per_energy;
+        const double t = static_cast<double>(waves) * (static_cast<double>(piece) * nc.fixed +
+                                                       static_cast<double>((piece + 255) / 256) * series);
         if (t < best) {
           best = t;
           nq = v;
@@ -453,7 +460,7 @@ int plan_create(int64_t ns, int64_t np, int64_t no, int64_t na, int mode, int pr
     delete p;
     return cuda_fail(e);
   }
-  Choice c = default_choice(prec, mode, no);
+  Choice c = default_choice(prec, mode);
   {
     std::lock_guard<std::mutex> lk(g_mu);
     auto it = g_tuned.find(key_of(dev, ns, np, no, na, mode, prec, want, p->n_bins));

@@ -23,6 +23,15 @@
 // FP64, the moments, the series and the rotations in the float-pair arithmetic of rad_df.cu
 // (products by FMA, Ogita-Rump-Oishi Dot2 sums), because GB300 executes FP64 at 1/64 of its FP32
 // rate: a float-pair multiply-add takes about a sixth of the time of an FP64 one.
+//
+// What bounds it: the FP64 pipe (79-90 % busy) in FP64; latency at 8 warps an SM in float pairs (255
+// registers a thread hold the moments; IPC 1.7). Measured, all kernels of a call, before (direct kernel
+// alone) and with it: one undulator, 4096 samples x 128 energies x 256 directions, FP64, 4.49 -> 0.60
+// ms; 64 sections of 500 samples x 192 log energies x 324 directions, spin 1/2, FP64, 80.9 -> 39.1 ms
+// (the 64 highest energies stay direct: 25.7 ms of it); 20 undulator periods, 40960 samples x 500
+// energies x 225 directions, float pairs, 21.6 -> 5.2 ms; 6 positrons x 12000 samples x 384 log energies
+// x 576 directions, spin 1/2, float pairs, 108 -> 57 ms. Tried and slower: 28 moments for spin 1/2 (41.1
+// against 39.6 ms, and spills in float pairs), 24 for the other models (5.6 -> 7.2 ms).
 #include <type_traits>
 
 #include "rad_df_reduce.cuh"
@@ -431,11 +440,16 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
             asm volatile("cp.async.commit_group;" ::: "memory");
           };
           fetch(warp, 0);
-          int slot = 0;
+          int slot = 0, terms_next = warp < ne ? n_terms[warp] : 0;
+          double ws_next = warp < ne ? wsv[warp] : 0.0;
           for (int e = warp; e < ne; e += kW, slot ^= 1) {
             fetch(e + kW, slot ^ 1);
-            const int terms = n_terms[e];
-            const double phi = __dmul_rn(wsv[e], Ac);
+            const int terms = terms_next;
+            const double phi = __dmul_rn(ws_next, Ac);
+            if (e + kW < ne) {
+              terms_next = n_terms[e + kW];
+              ws_next = wsv[e + kW];
+            }
             T sn, cs;
             float4 entry;
             float xh, xl;
@@ -581,8 +595,8 @@ NodeCost cheb_cost(int mode, bool df, int direct_gran) {
   c.cap = kWin;
   c.reach = 0.8f * 2.f * static_cast<float>(spin ? Cheb<RAD_SPIN_HALF>::kPhi : Cheb<RAD_CLASSICAL>::kPhi);
   c.direct = df ? (spin ? 1.25f : 1.05f) : (spin ? 10.2f : 9.2f);
-  c.fixed = df ? 26.f : 60.f;
-  c.per_energy = df ? 6.f : (spin ? 40.f : 35.f);
+  c.fixed = df ? 18.f : 60.f;
+  c.per_energy = df ? 4.f : (spin ? 40.f : 35.f);
   return c;
 }
 
