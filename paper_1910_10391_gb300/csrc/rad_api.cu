@@ -89,11 +89,12 @@ ShapeKey key_of(int dev, int64_t ns, int64_t np, int64_t no, int64_t na, int mod
 // 64 x 64 directions, 32 particles per launch). The mixed kernel runs 8 warps per block, 2 blocks
 // per SM; spin-1/2 keeps every sin/cos on the SFU, classical and spin-0 (two fewer sums per term)
 // take 1/8 of them on the FMA pipe. k_df's blocks of 4 warps take 128 energies of one
-// direction: the moment kernel takes the lowest ones in steps of as many, and 256 per block (3 % fewer
-// instructions per term) left half of a block idle for the 128 highest of 384.
-Choice default_choice(int precision, int mode) {
+// direction: the moment kernel takes the lowest ones in steps of as many, and 256 per block (3 to 5 %
+// faster per term, and taken where one such block holds all energies) left half of a block idle for the
+// 128 highest of 384.
+Choice default_choice(int precision, int mode, int64_t n_omega) {
   if (precision == RAD_FP64) return Choice{2, 8, 64, 1, 0};
-  if (precision == RAD_FP64_DF) return Choice{1, 4, 64, 1, 0};
+  if (precision == RAD_FP64_DF) return Choice{n_omega > 128 && n_omega <= 256 ? 2 : 1, 4, 64, 1, 0};
   if (mode == RAD_SPIN_HALF) return Choice{2, 8, 256, 1, 1, 0};
   return Choice{2, 8, 256, 1, 1, 6};
 }
@@ -116,7 +117,8 @@ constexpr int64_t kChebMinFp64 = 24, kChebMinDf = 64;
 constexpr int64_t kChebPartials = int64_t(1) << 26;
 
 // Work decomposition for a choice; (re)allocates scratch when it grows.
-int configure(rad_plan p, const Choice &c) {
+// `moments` false: without the moment kernel, whose finer split needs larger partials.
+int configure(rad_plan p, const Choice &c, bool moments = true) {
   if (!supported(p->precision, c)) return RAD_EINVAL;
   LaunchShape sh{c.R, c.NW, c.T, 0, 0, c.pe};
   const int occ = p->precision == RAD_FP64      ? occupancy_fp64(sh, p->mode)
@@ -142,10 +144,10 @@ int configure(rad_plan p, const Choice &c) {
   const bool per_particle = (p->want & RAD_PER_PARTICLE) != 0;
   // the node and moment forms go with the default launch shape; a caller that sets another asks for
   // that direct kernel
-  const Choice def = default_choice(p->precision, p->mode);
+  const Choice def = default_choice(p->precision, p->mode, p->n_omega);
   const bool def_shape = c.R == def.R && c.NW == def.NW && c.T == def.T && c.pp == def.pp;
   const bool df = p->precision == RAD_FP64_DF;
-  bool cheb = p->precision != RAD_MIXED && def_shape && p->n_omega >= (df ? kChebMinDf : kChebMinFp64) &&
+  bool cheb = moments && p->precision != RAD_MIXED && def_shape && p->n_omega >= (df ? kChebMinDf : kChebMinFp64) &&
               p->n_omega <= INT32_MAX && p->n_angles >= 16 && p->n_particles > 0;
   const int cheb_occ = cheb ? occupancy_cheb(p->mode, df) : 0;
   cheb = cheb_occ > 0;
@@ -189,7 +191,7 @@ int configure(rad_plan p, const Choice &c) {
         const int64_t waves = (v * p->n_particles * ctiles + slots - 1) / slots, piece = (avg_len + v - 1) / v;
         const double series = static_cast<double>(std::min<int64_t>(p->n_omega, nc.tile)) * nc.per_energy;
         const double t = static_cast<double>(waves) * (static_cast<double>(piece) * nc.fixed +
-                                                       static_cast<double>((piece + 255) / 256) * series);
+                                                       static_cast<double>((piece + 255) / 256) * (nc.per_run + series));
         if (t < best) {
           best = t;
           nq = v;
@@ -228,7 +230,7 @@ int configure(rad_plan p, const Choice &c) {
                                        : cheb && ctiles <= (INT32_MAX - 65536) / p->n_chunks;
   if (p->precision != RAD_MIXED && p->nodes) {
     p->cheb_grid = static_cast<int>(std::min<int64_t>(ctiles * p->n_chunks, cheb_res));
-    const size_t bytes = cheb_scratch_bytes(p->mode, p->cheb_grid);
+    const size_t bytes = cheb_scratch_bytes(p->mode, p->n_omega, p->cheb_grid);
     if (bytes > p->cheb_cap) {
       if (p->cheb_scratch) cudaFree(p->cheb_scratch);
       p->cheb_scratch = nullptr;
@@ -248,6 +250,10 @@ int configure(rad_plan p, const Choice &c) {
     p->part = nullptr;
     p->part_cap = 0;
     cudaError_t e = cudaMalloc(&p->part, need * sizeof(double));
+    if (e != cudaSuccess && cheb) {  // no room for the finer split: the direct kernel alone
+      (void)cudaGetLastError();
+      return configure(p, c, false);
+    }
     if (e != cudaSuccess) return cuda_fail(e);
     p->part_cap = need;
   }
@@ -368,14 +374,19 @@ int execute(rad_plan p, const double *samples, const int64_t *offsets, const dou
   if (e != cudaSuccess) return cuda_fail(e);
   NodeCost nc;
   if (p->nodes && p->precision == RAD_MIXED) {
-    nc = node_cost(p->n_omega, p->shape.R);
+    nc = node_cost(p->mode, p->n_omega, p->shape.R);
+    const int64_t items = node_tiles(p->n_omega) * p->n_angles * p->n_chunks, slots = 4LL * p->sms;
+    if (items < slots) nc.scale(static_cast<float>(slots) / static_cast<float>(items));
   } else if (p->nodes) {
     const bool df = p->precision == RAD_FP64_DF;
     nc = cheb_cost(p->mode, df, 32 * p->shape.R * (df ? p->shape.NW : 1));
     // idle lanes of the last direction tile cost as much as the others
     const float waste = static_cast<float>((p->n_angles + 31) / 32 * 32) / static_cast<float>(p->n_angles);
-    nc.fixed *= waste;
-    nc.per_energy *= waste;
+    const int64_t items = cheb_tiles(p->mode, p->n_omega, p->n_angles) * p->n_chunks;
+    if (p->n_particles > 0)
+      nc.cap = static_cast<float>(std::max<int64_t>(std::min<int64_t>(256, p->n_samples_total / p->n_particles / p->n_q), 1));
+    const int64_t slots = df ? 2LL * p->sms : p->sms;
+    nc.scale(waste * (items < slots ? static_cast<float>(slots) / static_cast<float>(items) : 1.f));
   }
   e = launch_validate(P, d_omega, need_dom, bin_of_angle, nc, st);
   if (e != cudaSuccess) return cuda_fail(e);
@@ -460,7 +471,7 @@ int plan_create(int64_t ns, int64_t np, int64_t no, int64_t na, int mode, int pr
     delete p;
     return cuda_fail(e);
   }
-  Choice c = default_choice(prec, mode);
+  Choice c = default_choice(prec, mode, no);
   {
     std::lock_guard<std::mutex> lk(g_mu);
     auto it = g_tuned.find(key_of(dev, ns, np, no, na, mode, prec, want, p->n_bins));

@@ -125,18 +125,23 @@ struct Num<true> {
   }
 };
 
-// A block's scratch: amplitudes [tile][2 NP][32], particle sums S [tile][32], series coefficients
-// [tile][kM], w* [tile], number of terms [tile], and (DF) the float-pair sin/cos table.
+// A block's scratch for n energies (the tile, or all of the call's if fewer): amplitudes [n][2 NP][32],
+// particle sums S [n][32], series coefficients [n][kM], w* [n], number of terms [n] and (DF) the
+// float-pair sin/cos table; every part on 16 bytes.
 template <int MODE>
 struct Scratch {
   using C = Cheb<MODE>;
-  static constexpr size_t kAmp = 0;
-  static constexpr size_t kS = kAmp + size_t(C::kTile) * 2 * C::NP * 32 * 8;
-  static constexpr size_t kCoef = kS + size_t(C::kTile) * 32 * 8;
-  static constexpr size_t kWs = kCoef + size_t(C::kTile) * C::kM * 8;
-  static constexpr size_t kTerms = kWs + size_t(C::kTile) * 8;
-  static constexpr size_t kTab = kTerms + size_t(C::kTile) * 4;
-  static constexpr size_t kTotal = kTab + dfr::kTabN * 16;
+  size_t amp, s, coef, ws, terms, tab, total;
+  __host__ __device__ explicit Scratch(int64_t n_omega) {
+    const size_t n = (static_cast<size_t>(n_omega < C::kTile ? n_omega : C::kTile) + 3) / 4 * 4;
+    amp = 0;
+    s = amp + n * 2 * C::NP * 32 * 8;
+    coef = s + n * 32 * 8;
+    ws = coef + n * C::kM * 8;
+    terms = ws + n * 8;
+    tab = terms + n * 4;
+    total = tab + dfr::kTabN * 16;
+  }
 };
 
 template <int MODE>
@@ -152,9 +157,19 @@ struct Smem {
   static constexpr int kTotal = kMisc + 64;
 };
 
+// 1 / v for normal v: one cubic step from the hardware's 20-bit reciprocal
+__device__ __forceinline__ double rcp_step(double v) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
+  const double e = fma(-v, r, 1.0);
+  return fma(fma(e, e, e), r, r);
+}
+
 // (2 - delta_m0) (-1)^{m/2} J_m(z) for m < M into out (as T), and the number of terms above 1e-18,
-// rounded up to even. Power series below z = 1/2, Miller's backward recurrence normalised by
-// J_0 + 2 sum J_2k = 1 above (M. Abramowitz, I. A. Stegun, 9.12).
+// rounded up to even. Power series below z = 1/2 (ended where the terms pass 1e-18), Miller's backward
+// recurrence normalised by J_0 + 2 sum J_2k = 1 above (M. Abramowitz, I. A. Stegun, 9.12). One thread
+// per energy, once per energy tile and particle energy: an FP64 instruction costs the warp 64 clocks, so
+// there is no division in the loops.
 template <bool DF, int M>
 __device__ int bessel_row(double z, typename Num<DF>::T *out) {
   int terms = 2;
@@ -164,31 +179,41 @@ __device__ int bessel_row(double z, typename Num<DF>::T *out) {
     if (fabs(v) > 1e-18 && m + 1 > terms) terms = m + 1;
   };
   if (z < 0.5) {
+    // J_m = (z/2)^m / m! sum_k q^k / (k! (m+1)..(m+k)), q = -z^2/4: with 1/((m+1)..(m+6)) over a common
+    // denominator the sum is one quotient
     const double q = -0.25 * z * z;
     double lead = 1.0;  // (z/2)^m / m!
     for (int m = 0; m < M; ++m) {
-      double s = 1.0, t = 1.0;
-      for (int k = 1; k < 9; ++k) {
-        t *= q / (k * static_cast<double>(m + k));
-        s += t;
+      double num = 0.0, den = 1.0;  // Horner from k = 6: 1 + q/(1 (m+1)) (1 + q/(2 (m+2)) (...))
+      for (int k = 6; k >= 1; --k) {
+        // (num, den) <- value 1 + q / (k (m + k)) * (num_k / den_k), kept as a fraction
+        const double inner = k == 6 ? 1.0 : num, id = k == 6 ? 1.0 : den, f = static_cast<double>(k * (m + k));
+        den = f * id;
+        num = fma(q, inner, den);
       }
-      put(m, lead * s);
-      lead *= 0.5 * z / (m + 1);
+      const double j = lead < 1e-19 ? 0.0 : lead * (num * rcp_step(den));
+      put(m, j);
+      lead *= 0.5 * z * rcp_step(m + 1.0);
+      if (lead < 1e-19) {
+        for (int i = m + 1; i < M; ++i) out[i] = Num<DF>::from(0.0);
+        break;
+      }
     }
   } else {
     const double rz = 2.0 / z;
     // twice: the normalising sum first, then the values (no array of them)
+    constexpr int kStart = M + 24;
     double hi = 0.0, lo = 1e-200, sum = 0.0;
-    for (int m = 60; m > 0; --m) {
+    for (int m = kStart; m > 0; --m) {
       const double t = fma(m * rz, lo, -hi);  // J_{m-1}
       hi = lo;
       lo = t;
-      if ((m - 1) % 2 == 0) sum += (m - 1 ? 2.0 : 1.0) * t;
+      if ((m - 1) % 2 == 0) sum += t;
     }
-    const double scale = 1.0 / sum;
+    const double scale = 1.0 / (2.0 * sum - lo);
     hi = 0.0;
     lo = 1e-200;
-    for (int m = 60; m > 0; --m) {
+    for (int m = kStart; m > 0; --m) {
       const double t = fma(m * rz, lo, -hi);
       hi = lo;
       lo = t;
@@ -205,7 +230,6 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
   using T = typename N::T;
   using A = typename N::A;
   using SM = Smem<MODE>;
-  using SC = Scratch<MODE>;
   constexpr int NP = C::NP, kM = C::kM, kTile = C::kTile;
   constexpr int NC = C::kSpin ? 8 : 6;
   static_assert(sizeof(T) == 8 && sizeof(A) == 8, "8-byte numbers");
@@ -222,13 +246,14 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
   if (s_item[1] != 0) return;
   const int64_t cut = *P.node_cut;  // energies [0, cut) are summed here, the others by the direct kernel
   if (cut <= 0) return;
-  unsigned char *scr = scratch_all + static_cast<size_t>(blockIdx.x) * SC::kTotal;
-  A *amp = reinterpret_cast<A *>(scr + SC::kAmp);
-  double *Ssum = reinterpret_cast<double *>(scr + SC::kS);
-  T *coef = reinterpret_cast<T *>(scr + SC::kCoef);
-  double *wsv = reinterpret_cast<double *>(scr + SC::kWs);
-  int *n_terms = reinterpret_cast<int *>(scr + SC::kTerms);
-  float4 *tab = reinterpret_cast<float4 *>(scr + SC::kTab);
+  const Scratch<MODE> sc(P.n_omega);
+  unsigned char *scr = scratch_all + static_cast<size_t>(blockIdx.x) * sc.total;
+  A *amp = reinterpret_cast<A *>(scr + sc.amp);
+  double *Ssum = reinterpret_cast<double *>(scr + sc.s);
+  T *coef = reinterpret_cast<T *>(scr + sc.coef);
+  double *wsv = reinterpret_cast<double *>(scr + sc.ws);
+  int *n_terms = reinterpret_cast<int *>(scr + sc.terms);
+  float4 *tab = reinterpret_cast<float4 *>(scr + sc.tab);
   if (DF)
     for (int i = tid; i < dfr::kTabN; i += kW * 32) tab[i] = dfr::table_pair(P.table[2 * i]);
 
@@ -363,12 +388,7 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
             const double x = fma(-nys, o[3], fma(-nxs, o[2], fma(-inv_a, o[1], fma(cns, o[0], off_x))));
             const double vx = o[4], vy = o[5];
             const double D = cn - o[9] - nx * vx - ny * vy;  // 1 - n.beta (Sec. II, g)
-            // 1 / D by one cubic step from the hardware's 20-bit reciprocal
-            double r;
-            asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(D));
-            const double eps = fma(-D, r, 1.0);
-            r = fma(fma(eps, eps, eps), r, r);
-            const double g = r * r;
+            const double r = rcp_step(D), g = r * r;
             const double a = nx - vx, b = ny - vy;
             const double mm = fma(ny, o[7], fma(nx, o[6], o[8]));  // n.beta_dot, weighted
             T f[NP];
@@ -579,24 +599,24 @@ int occupancy_cheb(int mode, bool df) {
   return e == cudaSuccess ? nb : 0;
 }
 
-size_t cheb_scratch_bytes(int mode, int grid) {
+size_t cheb_scratch_bytes(int mode, int64_t n_omega, int grid) {
   return static_cast<size_t>(grid) *
-         (mode == RAD_SPIN_HALF ? Scratch<RAD_SPIN_HALF>::kTotal : Scratch<RAD_CLASSICAL>::kTotal);
+         (mode == RAD_SPIN_HALF ? Scratch<RAD_SPIN_HALF>(n_omega).total : Scratch<RAD_CLASSICAL>(n_omega).total);
 }
 
-// Cost per sample and direction in SM clocks, for the choice of the cut (measured rates of the
-// kernels): per energy summed directly; per sample for the moments; per energy and run for the
-// series; reach: the phase range of a run.
+// Cost per sample and direction in SM clocks, for the choice of the cut, from the measured rates of the
+// kernels (direct: 1.3e8 and 4.6e9 terms; moments: the cases in the header).
 NodeCost cheb_cost(int mode, bool df, int direct_gran) {
   NodeCost c;
   const bool spin = mode == RAD_SPIN_HALF;
   c.gran = direct_gran;
   c.tile = cheb_tile(mode);
   c.cap = kWin;
-  c.reach = 0.8f * 2.f * static_cast<float>(spin ? Cheb<RAD_SPIN_HALF>::kPhi : Cheb<RAD_CLASSICAL>::kPhi);
-  c.direct = df ? (spin ? 1.25f : 1.05f) : (spin ? 10.2f : 9.2f);
-  c.fixed = df ? 18.f : 60.f;
-  c.per_energy = df ? 4.f : (spin ? 40.f : 35.f);
+  c.reach = 0.95f * 2.f * static_cast<float>(spin ? Cheb<RAD_SPIN_HALF>::kPhi : Cheb<RAD_CLASSICAL>::kPhi);
+  c.direct = df ? (spin ? 1.45f : 1.3f) : (spin ? 11.5f : 9.6f);
+  c.fixed = df ? (spin ? 36.f : 32.f) : 85.f;
+  c.per_run = df ? 20.f : 110.f;
+  c.per_energy = df ? (spin ? 17.f : 14.f) : (spin ? 58.f : 50.f);
   return c;
 }
 

@@ -109,12 +109,13 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 5 : 2) k_df(const Params P)
   float4 *sFa = reinterpret_cast<float4 *>(sm + L::kNk + T * 8);   // (fx_hi, fx_lo, fy_hi, fy_lo)
   float2 *sFj = reinterpret_cast<float2 *>(sm + L::kNk + T * 24);  // (j_hi, j_lo), spin 1/2 only
 
-  // energies below node_cut (a multiple of NW 32 R, or all of them) are summed by k_cheb
-  const int64_t cut = P.node_cut ? *P.node_cut : 0;
-  const int wt0 = static_cast<int>((cut + NW * 32 * R - 1) / (NW * 32 * R)), n_wt = P.n_wt - wt0;
-  if (n_wt <= 0) return;
-  const int64_t per_chunk = static_cast<int64_t>(n_wt) * P.n_nt;
-  const int64_t n_items = per_chunk * P.n_chunks;
+  // energies below node_cut (a multiple of NW 32 R, or all of them) are summed by k_cheb; read again for each
+  // item, so that nothing of it stays in registers through the term loop
+  auto first_tile = [&]() -> int {
+    const int64_t cut = P.node_cut ? *P.node_cut : 0;
+    return static_cast<int>((cut + NW * 32 * R - 1) / (NW * 32 * R));
+  };
+  if (first_tile() >= P.n_wt) return;
   int s = 0;
 
   for (;;) {
@@ -122,7 +123,9 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 5 : 2) k_df(const Params P)
     __syncthreads();
     const int64_t item = s_item[0];
     __syncthreads();
-    if (item >= n_items) break;
+    const int wt0 = first_tile(), n_wt = P.n_wt - wt0;
+    const int64_t per_chunk = static_cast<int64_t>(n_wt) * P.n_nt;
+    if (item >= per_chunk * P.n_chunks) break;
     const int64_t chunk = item / per_chunk;
     const int64_t rem = item % per_chunk;
     // one direction per item, shared by the block's warps (the per-sample preparation is done

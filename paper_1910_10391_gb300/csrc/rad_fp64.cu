@@ -78,12 +78,13 @@ __global__ void __launch_bounds__(NW * 32) k_fp64(const Params P) {
   double *myFx = myA + T, *myFy = myA + 2 * T;
   double *myJ = myA + 3 * T;  // spin-1/2 only
 
-  // energies below node_cut (a multiple of 32 R, or all of them) are summed by k_cheb
-  const int64_t cut = P.node_cut ? *P.node_cut : 0;
-  const int wt0 = static_cast<int>((cut + 32 * R - 1) / (32 * R)), n_wt = P.n_wt - wt0;
-  if (n_wt <= 0) return;
-  const int64_t per_chunk = static_cast<int64_t>(n_wt) * P.n_nt;
-  const int64_t n_items = per_chunk * P.n_chunks;
+  // energies below node_cut (a multiple of 32 R, or all of them) are summed by k_cheb; read again for each
+  // item, so that nothing of it stays in registers through the term loop
+  auto first_tile = [&]() -> int {
+    const int64_t cut = P.node_cut ? *P.node_cut : 0;
+    return static_cast<int>((cut + 32 * R - 1) / (32 * R));
+  };
+  if (first_tile() >= P.n_wt) return;
   int s = 0;  // stage of the next tile to consume
 
   for (;;) {
@@ -91,7 +92,9 @@ __global__ void __launch_bounds__(NW * 32) k_fp64(const Params P) {
     __syncthreads();
     const int64_t item = s_item[0];
     __syncthreads();
-    if (item >= n_items) break;
+    const int wt0 = first_tile(), n_wt = P.n_wt - wt0;
+    const int64_t per_chunk = static_cast<int64_t>(n_wt) * P.n_nt;
+    if (item >= per_chunk * P.n_chunks) break;
     const int64_t chunk = item / per_chunk;
     const int64_t rem = item % per_chunk;
     const int nt = static_cast<int>(rem / n_wt), wt = wt0 + static_cast<int>(rem % n_wt);

@@ -259,13 +259,20 @@ cudaError_t launch_mixed_pp(const Params &P, const float *prep, LaunchShape *sha
 bool node_path_allowed(const LaunchShape &s, int64_t n_omega, int64_t n_angles, int64_t n_chunks);
 // Chooses on the device how many of the lowest energies the node (or moment) kernel takes. Costs per
 // sample and direction in SM clocks: `direct` per energy summed directly; `fixed` per tile of `tile`
-// energies and `per_energy` per energy over the run length, which is the number of samples within a
-// phase range of `reach` radians over the tile's span of w*, at most `cap`.
+// energies, and `per_run` and `per_energy` per energy over the run length, which is the number of samples
+// within a phase range of `reach` radians over the tile's span of w*, at most `cap`.
 struct NodeCost {
   int gran = 64, tile = 512, from_zero = 1;
-  float direct = 0.f, fixed = 0.f, per_energy = 0.f, reach = 0.f, cap = 64.f;
+  float direct = 0.f, fixed = 0.f, per_run = 0.f, per_energy = 0.f, reach = 0.f, cap = 64.f;
+  // for a kernel that fills only a part of the SMs (or lanes) the costs rise by that factor
+  void scale(float f) {
+    fixed *= f;
+    per_run *= f;
+    per_energy *= f;
+  }
 };
-NodeCost node_cost(int64_t n_omega, int direct_r);
+NodeCost node_cost(int mode, int64_t n_omega, int direct_r);
+int64_t node_tiles(int64_t n_omega);  // energy tiles of the node kernel
 cudaError_t launch_mixed_nodes(const Params &P, const float *prep, int sms, cudaStream_t st);
 
 // FP64-accurate kernel with double-float FP32 arithmetic after the FP64 phase (rad_df.cu)
@@ -277,7 +284,7 @@ cudaError_t launch_df(const Params &P, LaunchShape *shape, cudaStream_t st);
 int64_t cheb_tiles(int mode, int64_t n_omega, int64_t n_angles);  // work items per chunk
 int cheb_tile(int mode);                                          // energies per tile
 int occupancy_cheb(int mode, bool df);
-size_t cheb_scratch_bytes(int mode, int grid);
+size_t cheb_scratch_bytes(int mode, int64_t n_omega, int grid);
 NodeCost cheb_cost(int mode, bool df, int direct_gran);
 cudaError_t launch_cheb(const Params &P, bool df, unsigned char *scratch, int grid, cudaStream_t st);
 

@@ -581,19 +581,23 @@ bool node_path_allowed(const LaunchShape &s, int64_t n_omega, int64_t n_angles, 
 }
 
 // Runs reach 56 pi of phase range over the tile's span, three quarters of it on average (they are
-// powers of two).
-NodeCost node_cost(int64_t n_omega, int direct_r) {
+// powers of two). Costs from the measured rates: 17.4 clocks per sample and direction of the 512-energy
+// ensemble (classical, runs of about 50), 52 of the 1024-energy batch (spin 1/2, two tiles).
+NodeCost node_cost(int mode, int64_t n_omega, int direct_r) {
+  const bool spin = mode == RAD_SPIN_HALF;
   NodeCost c;
   c.gran = 32 * direct_r;
   c.tile = 128 * node_r(n_omega);
   c.from_zero = 0;
-  c.direct = 1.0f / 8.5f;
-  c.fixed = 4.5f;
-  c.per_energy = 0.7f;
+  c.direct = spin ? 1.0f / 7.6f : 1.0f / 8.5f;
+  c.fixed = spin ? 9.5f : 6.5f;
+  c.per_energy = spin ? 1.45f : 0.95f;
   c.reach = static_cast<float>(0.75 * 56.0 * kPi);
   c.cap = 64.f;
   return c;
 }
+
+int64_t node_tiles(int64_t n_omega) { return (n_omega + 128 * node_r(n_omega) - 1) / (128 * node_r(n_omega)); }
 
 cudaError_t launch_mixed_nodes(const Params &P, const float *prep, int sms, cudaStream_t st) {
   const int r = node_r(P.n_omega);

@@ -174,12 +174,13 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? (R <= 2 ? 2 : 1) : 3) k_mix
   __syncthreads();
   uint32_t full_par[2] = {0u, 0u};   // consumers: next parity of full[s]
   uint32_t uses[2] = {0u, 0u};       // producer (thread 0): copies issued into stage s so far
-  // energies below node_cut (a multiple of 32 R, or all of them) are summed by k_mixed_nodes
-  const int64_t cut = P.node_cut ? *P.node_cut : 0;
-  const int wt0 = static_cast<int>((cut + 32 * R - 1) / (32 * R)), n_wt = P.n_wt - wt0;
-  const int64_t per_chunk = static_cast<int64_t>(n_wt) * P.n_nt;
-  const int64_t n_items = per_chunk * P.n_chunks;
-  if (n_wt <= 0) return;
+  // energies below node_cut (a multiple of 32 R, or all of them) are summed by k_mixed_nodes; read again for each
+  // item, so that nothing of it stays in registers through the term loop
+  auto first_tile = [&]() -> int {
+    const int64_t cut = P.node_cut ? *P.node_cut : 0;
+    return static_cast<int>((cut + 32 * R - 1) / (32 * R));
+  };
+  if (first_tile() >= P.n_wt) return;
   int s = 0;
 
   // thread 0: wait until every warp released stage st's previous tile, then fill it
@@ -200,7 +201,9 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? (R <= 2 ? 2 : 1) : 3) k_mix
     __syncthreads();
     const int64_t item = s_item[0];
     __syncthreads();
-    if (item >= n_items) break;
+    const int wt0 = first_tile(), n_wt = P.n_wt - wt0;
+    const int64_t per_chunk = static_cast<int64_t>(n_wt) * P.n_nt;
+    if (item >= per_chunk * P.n_chunks) break;
     const int64_t chunk = item / per_chunk;
     const int64_t rem = item % per_chunk;
     const int nt = static_cast<int>(rem / n_wt), wt = wt0 + static_cast<int>(rem % n_wt);
@@ -472,9 +475,11 @@ bool shape_supported_mixed_pp(int R, int NW, int T) {
 
 cudaError_t launch_prep_samples(const Params &P, int T, float *prep, cudaStream_t st) {
   if (P.n_particles == 0) return cudaSuccess;
-  // 256 samples per block up to 64 blocks per particle: one long trajectory has to spread over the SMs
-  const int64_t per = P.n_samples_total / P.n_particles / 256;
-  dim3 grd(static_cast<unsigned>(per < 8 ? 8 : per > 64 ? 64 : per), grid_y(P.n_particles));
+  // 8 blocks per particle; fewer particles than 76 get more, down to 256 samples each: one long trajectory
+  // has to spread over the SMs
+  const int64_t per = P.n_samples_total / P.n_particles / 256, most = 608 / P.n_particles;
+  const int64_t gx = per < most ? per : most;
+  dim3 grd(static_cast<unsigned>(gx < 8 ? 8 : gx > 64 ? 64 : gx), grid_y(P.n_particles));
   k_prep_samples<<<grd, 256, 0, st>>>(P, T, prep);
   return cudaGetLastError();
 }
