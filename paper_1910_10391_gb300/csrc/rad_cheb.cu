@@ -612,6 +612,7 @@ NodeCost cheb_cost(int mode, bool df, int direct_gran) {
   c.gran = direct_gran;
   c.tile = cheb_tile(mode);
   c.cap = kWin;
+  c.widen = 1.6f;  // the widest of 32 directions, a row or more of a grid
   c.reach = 0.95f * 2.f * static_cast<float>(spin ? Cheb<RAD_SPIN_HALF>::kPhi : Cheb<RAD_CLASSICAL>::kPhi);
   c.direct = df ? (spin ? 1.45f : 1.3f) : (spin ? 11.5f : 9.6f);
   c.fixed = df ? (spin ? 36.f : 32.f) : 85.f;

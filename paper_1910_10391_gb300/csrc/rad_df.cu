@@ -89,7 +89,13 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 5 : 2) k_df(const Params P)
   int *s_item = reinterpret_cast<int *>(sm + L::kMisc);
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) s_item[1] = *reinterpret_cast<volatile int *>(P.status);
+  // energies below node_cut (a multiple of NW 32 R, or all of them) are summed by k_cheb; the first tile above
+  // it stays in shared memory, out of the term loop's registers
+  if (tid == 0) {
+    const int64_t cut = P.node_cut ? *P.node_cut : 0;
+    s_item[1] = *reinterpret_cast<volatile int *>(P.status);
+    s_item[2] = static_cast<int>((cut + NW * 32 * R - 1) / (NW * 32 * R));
+  }
   __syncthreads();
   if (s_item[1] != 0) return;
 
@@ -109,13 +115,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 5 : 2) k_df(const Params P)
   float4 *sFa = reinterpret_cast<float4 *>(sm + L::kNk + T * 8);   // (fx_hi, fx_lo, fy_hi, fy_lo)
   float2 *sFj = reinterpret_cast<float2 *>(sm + L::kNk + T * 24);  // (j_hi, j_lo), spin 1/2 only
 
-  // energies below node_cut (a multiple of NW 32 R, or all of them) are summed by k_cheb; read again for each
-  // item, so that nothing of it stays in registers through the term loop
-  auto first_tile = [&]() -> int {
-    const int64_t cut = P.node_cut ? *P.node_cut : 0;
-    return static_cast<int>((cut + NW * 32 * R - 1) / (NW * 32 * R));
-  };
-  if (first_tile() >= P.n_wt) return;
+  if (s_item[2] >= P.n_wt) return;
   int s = 0;
 
   for (;;) {
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 5 : 2) k_df(const Params P)
     __syncthreads();
     const int64_t item = s_item[0];
     __syncthreads();
-    const int wt0 = first_tile(), n_wt = P.n_wt - wt0;
+    const int wt0 = s_item[2], n_wt = P.n_wt - wt0;
     const int64_t per_chunk = static_cast<int64_t>(n_wt) * P.n_nt;
     if (item >= per_chunk * P.n_chunks) break;
     const int64_t chunk = item / per_chunk;

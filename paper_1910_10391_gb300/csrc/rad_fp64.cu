@@ -62,7 +62,13 @@ __global__ void __launch_bounds__(NW * 32) k_fp64(const Params P) {
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // a failed device data check skips the computation (one read per block, shared by all threads)
-  if (tid == 0) s_item[1] = *reinterpret_cast<volatile int *>(P.status);
+  // energies below node_cut (a multiple of 32 R, or all of them) are summed by k_cheb; the first tile above
+  // it stays in shared memory, out of the term loop's registers
+  if (tid == 0) {
+    const int64_t cut = P.node_cut ? *P.node_cut : 0;
+    s_item[1] = *reinterpret_cast<volatile int *>(P.status);
+    s_item[2] = static_cast<int>((cut + 32 * R - 1) / (32 * R));
+  }
   __syncthreads();
   if (s_item[1] != 0) return;
 
@@ -78,13 +84,7 @@ __global__ void __launch_bounds__(NW * 32) k_fp64(const Params P) {
   double *myFx = myA + T, *myFy = myA + 2 * T;
   double *myJ = myA + 3 * T;  // spin-1/2 only
 
-  // energies below node_cut (a multiple of 32 R, or all of them) are summed by k_cheb; read again for each
-  // item, so that nothing of it stays in registers through the term loop
-  auto first_tile = [&]() -> int {
-    const int64_t cut = P.node_cut ? *P.node_cut : 0;
-    return static_cast<int>((cut + 32 * R - 1) / (32 * R));
-  };
-  if (first_tile() >= P.n_wt) return;
+  if (s_item[2] >= P.n_wt) return;
   int s = 0;  // stage of the next tile to consume
 
   for (;;) {
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(NW * 32) k_fp64(const Params P) {
     __syncthreads();
     const int64_t item = s_item[0];
     __syncthreads();
-    const int wt0 = first_tile(), n_wt = P.n_wt - wt0;
+    const int wt0 = s_item[2], n_wt = P.n_wt - wt0;
     const int64_t per_chunk = static_cast<int64_t>(n_wt) * P.n_nt;
     if (item >= per_chunk * P.n_chunks) break;
     const int64_t chunk = item / per_chunk;

@@ -260,10 +260,11 @@ bool node_path_allowed(const LaunchShape &s, int64_t n_omega, int64_t n_angles, 
 // Chooses on the device how many of the lowest energies the node (or moment) kernel takes. Costs per
 // sample and direction in SM clocks: `direct` per energy summed directly; `fixed` per tile of `tile`
 // energies, and `per_run` and `per_energy` per energy over the run length, which is the number of samples
-// within a phase range of `reach` radians over the tile's span of w*, at most `cap`.
+// within a phase range of `reach` radians over the tile's span of w*, at most `cap`, a power of two if
+// `pow2`; `widen`: a block's widest direction against the mean.
 struct NodeCost {
-  int gran = 64, tile = 512, from_zero = 1;
-  float direct = 0.f, fixed = 0.f, per_run = 0.f, per_energy = 0.f, reach = 0.f, cap = 64.f;
+  int gran = 64, tile = 512, from_zero = 1, pow2 = 0;
+  float widen = 1.f, direct = 0.f, fixed = 0.f, per_run = 0.f, per_energy = 0.f, reach = 0.f, cap = 64.f;
   // for a kernel that fills only a part of the SMs (or lanes) the costs rise by that factor
   void scale(float f) {
     fixed *= f;

@@ -580,8 +580,7 @@ bool node_path_allowed(const LaunchShape &s, int64_t n_omega, int64_t n_angles, 
   return n_angles <= (INT32_MAX - 65536) / tiles / n_chunks;  // the 32-bit work counter
 }
 
-// Runs reach 56 pi of phase range over the tile's span, three quarters of it on average (they are
-// powers of two). Costs from the measured rates: 17.4 clocks per sample and direction of the 512-energy
+// Runs reach 56 pi of phase range over the tile's span (twofold oversampling, 56 node spacings). Costs from the measured rates: 17.4 clocks per sample and direction of the 512-energy
 // ensemble (classical, runs of about 50), 52 of the 1024-energy batch (spin 1/2, two tiles).
 NodeCost node_cost(int mode, int64_t n_omega, int direct_r) {
   const bool spin = mode == RAD_SPIN_HALF;
@@ -590,9 +589,10 @@ NodeCost node_cost(int mode, int64_t n_omega, int direct_r) {
   c.tile = 128 * node_r(n_omega);
   c.from_zero = 0;
   c.direct = spin ? 1.0f / 7.6f : 1.0f / 8.5f;
-  c.fixed = spin ? 9.5f : 6.5f;
-  c.per_energy = spin ? 1.45f : 0.95f;
-  c.reach = static_cast<float>(0.75 * 56.0 * kPi);
+  c.fixed = spin ? 8.5f : 6.8f;
+  c.per_energy = spin ? 1.35f : 1.1f;
+  c.pow2 = 1;
+  c.reach = static_cast<float>(56.0 * kPi);
   c.cap = 64.f;
   return c;
 }

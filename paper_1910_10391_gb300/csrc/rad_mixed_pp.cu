@@ -161,7 +161,13 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? (R <= 2 ? 2 : 1) : 3) k_mix
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   float4 *myF = reinterpret_cast<float4 *>(sm + L::kNk + warp * L::kNkWarp);
 
-  if (tid == 0) s_item[1] = *reinterpret_cast<volatile int *>(P.status);
+  // energies below node_cut (a multiple of 32 R, or all of them) are summed by k_mixed_nodes; the first tile above
+  // it stays in shared memory, out of the term loop's registers
+  if (tid == 0) {
+    const int64_t cut = P.node_cut ? *P.node_cut : 0;
+    s_item[1] = *reinterpret_cast<volatile int *>(P.status);
+    s_item[2] = static_cast<int>((cut + 32 * R - 1) / (32 * R));
+  }
   __syncthreads();
   if (s_item[1] != 0) return;
   if (tid == 0) {
@@ -174,13 +180,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? (R <= 2 ? 2 : 1) : 3) k_mix
   __syncthreads();
   uint32_t full_par[2] = {0u, 0u};   // consumers: next parity of full[s]
   uint32_t uses[2] = {0u, 0u};       // producer (thread 0): copies issued into stage s so far
-  // energies below node_cut (a multiple of 32 R, or all of them) are summed by k_mixed_nodes; read again for each
-  // item, so that nothing of it stays in registers through the term loop
-  auto first_tile = [&]() -> int {
-    const int64_t cut = P.node_cut ? *P.node_cut : 0;
-    return static_cast<int>((cut + 32 * R - 1) / (32 * R));
-  };
-  if (first_tile() >= P.n_wt) return;
+  if (s_item[2] >= P.n_wt) return;
   int s = 0;
 
   // thread 0: wait until every warp released stage st's previous tile, then fill it
@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? (R <= 2 ? 2 : 1) : 3) k_mix
     __syncthreads();
     const int64_t item = s_item[0];
     __syncthreads();
-    const int wt0 = first_tile(), n_wt = P.n_wt - wt0;
+    const int wt0 = s_item[2], n_wt = P.n_wt - wt0;
     const int64_t per_chunk = static_cast<int64_t>(n_wt) * P.n_nt;
     if (item >= per_chunk * P.n_chunks) break;
     const int64_t chunk = item / per_chunk;

@@ -15,21 +15,23 @@ namespace {
 __device__ __forceinline__ bool finite_d(double v) { return isfinite(v); }
 
 // Chooses how many of the lowest energies go through the node or moment kernel (0: none), from the
-// trajectories' largest phase length per sample within windows of 256 (which bounds the kernels' runs;
-// its mean over windows, particles and directions) and the costs in c_ (see NodeCost). One block of 256
+// trajectories' largest phase length per sample within windows of 256 (which bounds the kernels' runs) and
+// the costs in c_ (see NodeCost). One block of 256
 // threads; the energies must ascend (else none). It runs beside the checks, so it trusts no input:
 // offsets outside the records count for nothing, and other bad values only move a cut that the
 // failed check keeps from being used.
 __device__ void node_plan(const Params &P, const NodeCost &c_) {
-  __shared__ float s_step[256], s_n[256];
+  __shared__ float s_sum[2][8];
   const int tid = threadIdx.x;
   bool bad = false;
   for (int64_t i = tid; i + 1 < P.n_omega; i += 256) bad |= !(P.hw[i] <= P.hw[i + 1]);
-  // 16 particles x 16 directions spread over the call, and of each one window, placed by the thread
+  // 256 directions in golden-ratio steps (a stride would fall on one column of a rectangular grid) and
+  // 16 particles spread over the call, and of each pair one window, placed by the thread
   float widest = 0.f, cnt = 0.f;
   if (P.n_particles > 0) {
     const int64_t p = (tid >> 4) * P.n_particles / 16;
-    const int64_t j = ((tid & 15) * P.n_angles + P.n_angles / 2) / 16;
+    const float gold = static_cast<float>(tid) * 0.618033989f;
+    const int64_t j = min(static_cast<int64_t>((gold - floorf(gold)) * static_cast<float>(P.n_angles)), P.n_angles - 1);
     const int64_t ka = P.offsets[p], kb = P.offsets[p + 1];
     if (ka >= 0 && kb - ka >= 2 && kb <= P.n_samples_total) {
       const double *a = P.samples + ka * kRec;
@@ -45,37 +47,46 @@ __device__ void node_plan(const Params &P, const NodeCost &c_) {
       cnt = 1.f;
     }
   }
-  s_step[tid] = widest;
-  s_n[tid] = cnt;
-  bad = __syncthreads_or(bad);
-  for (int o = 128; o > 0; o >>= 1) {
-    if (tid < o) {
-      s_step[tid] += s_step[tid + o];
-      s_n[tid] += s_n[tid + o];
-    }
+  // sum over the block, the same in every thread
+  int turn = 0;
+  auto block_sum = [&](float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((tid & 31) == 0) s_sum[turn][tid >> 5] = v;
     __syncthreads();
-  }
-  if (tid != 0 || bad || P.n_particles == 0) return;
-  // a kernel's block takes the widest of its directions: a sixth more than the mean
-  const float step = s_step[0] / s_n[0] * (7.0f / 6.0f);
+    float t = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) t += s_sum[turn][i];
+    turn ^= 1;
+    return t;
+  };
+  bad = __syncthreads_or(bad);
+  const float windows = block_sum(cnt);
+  if (bad || !(windows > 0.f)) return;
+  const float step = widest * c_.widen;
   const float inv_E = P.mode == RAD_CLASSICAL ? 0.f : static_cast<float>(1.0 / P.energy[0]);
   auto ws = [&](int64_t i) {  // FP32: an estimate, and an FP64 division would cost 1000 clocks here
     const float h = static_cast<float>(P.hw[i]);
     return h * static_cast<float>(1.0 / kHbarC) / (1.f - h * inv_E);
   };
   // the route has to promise a fifth less than the direct sum: the estimate is that good (over 110 drawn
-  // calls of the library's ranges the slowest came out 6 % slower than directly at 15 %)
+  // calls of the library's ranges the slowest came out 7 % slower than directly, a call of half a ms)
   float best = 0.8f * c_.direct * static_cast<float>(P.n_omega), done = 0.f;  // done: whole tiles below
-  const int64_t gran = c_.gran, tile = c_.tile;
+  // at most some hundred steps: beyond 64 tiles whole groups of them are taken at once
+  const int64_t group = (P.n_omega + 64 * static_cast<int64_t>(c_.tile) - 1) / (64 * static_cast<int64_t>(c_.tile));
+  const int64_t tile = c_.tile * group, gran = group > 1 ? tile : c_.gran;
   int64_t cut = 0;
   float lo = 0.f;
   for (int64_t e = 0; e < P.n_omega; e += gran) {
     const int64_t t0 = e / tile * tile;
     const int64_t end = e + gran < P.n_omega ? e + gran : P.n_omega;
     if (e == t0) lo = c_.from_zero ? 0.f : ws(t0);
-    const float span = (ws(end - 1) - lo) * step;
-    const float runlen = fminf(fmaxf(c_.reach / fmaxf(span, 1e-30f), 1.f), c_.cap);
-    const float part = c_.fixed + (c_.per_run + c_.per_energy * static_cast<float>(end - t0)) / runlen;
+    // runs per sample, the mean over the windows
+    float runlen = fminf(fmaxf(c_.reach / fmaxf((ws(end - 1) - lo) * step, 1e-30f), 1.f), c_.cap);
+    if (c_.pow2) runlen = exp2f(floorf(log2f(runlen)));
+    const float runs = block_sum(cnt > 0.f ? 1.f / runlen : 0.f) / windows;
+    const float tiles = static_cast<float>(group);
+    const float part = tiles * c_.fixed + (tiles * c_.per_run + c_.per_energy * static_cast<float>(end - t0)) * runs;
     const float total = done + part + c_.direct * static_cast<float>(P.n_omega - end);
     if (total < best) {
       best = total;
@@ -83,7 +94,7 @@ __device__ void node_plan(const Params &P, const NodeCost &c_) {
     }
     if (end == t0 + tile) done += part;
   }
-  *P.node_cut = static_cast<int>(cut);
+  if (tid == 0) *P.node_cut = static_cast<int>(cut);
 }
 
 // One grid-stride pass over every device input; any violation sets RAD_EDATA.
