@@ -273,6 +273,24 @@ int rad_plan_set_prepass(rad_plan plan, int enable);
 int rad_plan_set_sincos_split(rad_plan plan, int every);
 
 /*
+ * rad_plan_set_cut -- how many of the lowest photon energies are summed over runs of samples
+ * (RAD_MIXED: equispaced frequency nodes; RAD_FP64, RAD_FP64_DF: Chebyshev moments) instead of
+ * term by term. n_lowest = -1 (a new plan's setting): chosen on the device in every call, from
+ * the kernels' costs. 0: none. Otherwise n_omega or a multiple of the energies of one work
+ * item of the term-by-term kernel (32 R; RAD_FP64_DF 32 R NW). It applies while the
+ * plan has the launch shape that a new plan of its size has; energies that do not ascend are
+ * summed term by term whatever is set. RAD_EINVAL for other values, and for n_lowest > 0
+ * where the plan has no such kernel: RAD_MIXED below 96 energies or without its pre-pass,
+ * RAD_FP64 below 24 and RAD_FP64_DF below 64 energies, both below 16 directions or without
+ * particles, and other launch shapes (the plan is unchanged). May reallocate scratch, as
+ * rad_plan_set_shape. rad_plan_describe shows it as cut=auto, cut=0 or the number.
+ * rad_plan_last_cut -- the number of the last execute (waits for the device), RAD_EINVAL before
+ * the first one.
+ */
+int rad_plan_set_cut(rad_plan plan, int64_t n_lowest);
+int rad_plan_last_cut(rad_plan plan, int64_t *n_lowest);
+
+/*
  * rad_plan_set_phase_budget -- RAD_MIXED plans only: the error-budget guard's limit, in radians
  * (default 8192). Every RAD_MIXED call bounds its in-tile phase offsets on the device,
  *   X = max over particles and samples of w*_max (c_max |t_k - t_ref| + |dz_k - dz_ref|

@@ -205,6 +205,10 @@ def load(build_if_missing: bool = True):
         lib.rad_plan_set_sincos_split.restype = c_int
         lib.rad_plan_set_phase_budget.argtypes = [P, ctypes.c_double]
         lib.rad_plan_set_phase_budget.restype = c_int
+        lib.rad_plan_set_cut.argtypes = [P, i64]
+        lib.rad_plan_set_cut.restype = c_int
+        lib.rad_plan_last_cut.argtypes = [P, ctypes.POINTER(i64)]
+        lib.rad_plan_last_cut.restype = c_int
         lib.rad_plan_describe.argtypes = [P, ctypes.c_char_p, c_int]
         lib.rad_plan_describe.restype = c_int
         lib.rad_plan_set_timing.argtypes = [P, c_int]
@@ -612,6 +616,16 @@ class Plan:
 
     def set_phase_budget(self, radians) -> int:
         return load().rad_plan_set_phase_budget(self._h, float(radians))
+
+    def set_cut(self, n_lowest=-1) -> int:
+        return load().rad_plan_set_cut(self._h, int(n_lowest))
+
+    def last_cut(self) -> int:
+        v = ctypes.c_int64()
+        rc = load().rad_plan_last_cut(self._h, ctypes.byref(v))
+        if rc:
+            raise RadError(rc, "rad_plan_last_cut")
+        return v.value
 
     def describe(self) -> str:
         buf = ctypes.create_string_buffer(512)

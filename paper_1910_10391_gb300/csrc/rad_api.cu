@@ -50,6 +50,8 @@ struct rad_plan_s {
   LaunchShape shape{};
   int n_wt = 0, n_nt = 0, amp_mode = 0, n_q = 1;
   bool nodes = false;  // the lowest energies may go through the frequency-node or moment kernel
+  int64_t set_cut = -1;  // how many of them: as asked for (rad_plan_set_cut), or by the costs (-1)
+  bool ran = false;
   int cheb_grid = 0;   // resident blocks of the moment kernel (FP64 forms)
   unsigned char *cheb_scratch = nullptr;
   size_t cheb_cap = 0;
@@ -117,7 +119,7 @@ constexpr int64_t kChebMinFp64 = 24, kChebMinDf = 64;
 constexpr int64_t kChebPartials = int64_t(1) << 26;
 
 // Work decomposition for a choice; (re)allocates scratch when it grows.
-// `moments` false: without the moment kernel, whose finer split needs larger partials.
+// `moments` false: without the node or moment kernel.
 int configure(rad_plan p, const Choice &c, bool moments = true) {
   if (!supported(p->precision, c)) return RAD_EINVAL;
   LaunchShape sh{c.R, c.NW, c.T, 0, 0, c.pe};
@@ -147,6 +149,7 @@ int configure(rad_plan p, const Choice &c, bool moments = true) {
   const Choice def = default_choice(p->precision, p->mode, p->n_omega);
   const bool def_shape = c.R == def.R && c.NW == def.NW && c.T == def.T && c.pp == def.pp;
   const bool df = p->precision == RAD_FP64_DF;
+  moments &= p->set_cut != 0;
   bool cheb = moments && p->precision != RAD_MIXED && def_shape && p->n_omega >= (df ? kChebMinDf : kChebMinFp64) &&
               p->n_omega <= INT32_MAX && p->n_angles >= 16 && p->n_particles > 0;
   const int cheb_occ = cheb ? occupancy_cheb(p->mode, df) : 0;
@@ -226,7 +229,7 @@ int configure(rad_plan p, const Choice &c, bool moments = true) {
   sh.grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(p->n_items, resident)));
   p->shape = sh;
   p->choice = c;
-  p->nodes = p->precision == RAD_MIXED ? c.pp && def_shape && node_path_allowed(sh, p->n_omega, p->n_angles, p->n_chunks)
+  p->nodes = p->precision == RAD_MIXED ? moments && c.pp && def_shape && node_path_allowed(sh, p->n_omega, p->n_angles, p->n_chunks)
                                        : cheb && ctiles <= (INT32_MAX - 65536) / p->n_chunks;
   if (p->precision != RAD_MIXED && p->nodes) {
     p->cheb_grid = static_cast<int>(std::min<int64_t>(ctiles * p->n_chunks, cheb_res));
@@ -264,11 +267,11 @@ int configure(rad_plan p, const Choice &c, bool moments = true) {
   char buf[256];
   std::snprintf(buf, sizeof buf,
                 "precision=%s mode=%d R=%d NW=%d T=%d grid=%d occ=%d items=%lld chunks=%lld amp=%d nq=%d pp=%d "
-                "pe=%d",
+                "pe=%d cut=%s",
                 p->precision == RAD_FP64 ? "fp64" : p->precision == RAD_FP64_DF ? "fp64_df" : "mixed", p->mode, c.R,
                 c.NW, c.T, sh.grid, occ,
                 static_cast<long long>(p->n_items), static_cast<long long>(p->n_chunks), p->amp_mode,
-                p->n_q, c.pp, c.pe);
+                p->n_q, c.pp, c.pe, !p->nodes ? "0" : p->set_cut < 0 ? "auto" : std::to_string(p->set_cut).c_str());
   p->desc = buf;
   return RAD_OK;
 }
@@ -388,6 +391,8 @@ int execute(rad_plan p, const double *samples, const int64_t *offsets, const dou
     const int64_t slots = df ? 2LL * p->sms : p->sms;
     nc.scale(waste * (items < slots ? static_cast<float>(slots) / static_cast<float>(items) : 1.f));
   }
+  nc.set_cut = p->set_cut;
+  p->ran = true;
   e = launch_validate(P, d_omega, need_dom, bin_of_angle, nc, st);
   if (e != cudaSuccess) return cuda_fail(e);
   LaunchShape sh = p->shape;
@@ -597,6 +602,33 @@ int rad_plan_set_sincos_split(rad_plan plan, int every) {
   int rc = configure(plan, c);
   if (rc) configure(plan, old);
   return rc;
+}
+
+int rad_plan_set_cut(rad_plan plan, int64_t n_lowest) {
+  if (!plan || n_lowest < -1 || n_lowest > plan->n_omega) return RAD_EINVAL;
+  const int64_t gran = 32LL * plan->choice.R * (plan->precision == RAD_FP64_DF ? plan->choice.NW : 1);
+  if (n_lowest > 0 && n_lowest < plan->n_omega && n_lowest % gran != 0) return RAD_EINVAL;
+  const int64_t old = plan->set_cut;
+  plan->set_cut = n_lowest;
+  int rc = configure(plan, plan->choice);
+  if (!rc && n_lowest > 0 && !plan->nodes) rc = RAD_EINVAL;
+  if (rc) {
+    plan->set_cut = old;
+    configure(plan, plan->choice);
+  }
+  return rc;
+}
+
+int rad_plan_last_cut(rad_plan plan, int64_t *n_lowest) {
+  if (!plan || !n_lowest || !plan->ran) return RAD_EINVAL;
+  int v = 0;
+  if (plan->nodes) {
+    cudaError_t e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = cudaMemcpy(&v, plan->ctrl + 2, sizeof(int), cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return cuda_fail(e);
+  }
+  *n_lowest = v;
+  return RAD_OK;
 }
 
 int rad_plan_set_phase_budget(rad_plan plan, double radians) {

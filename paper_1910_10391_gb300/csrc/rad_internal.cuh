@@ -264,6 +264,7 @@ bool node_path_allowed(const LaunchShape &s, int64_t n_omega, int64_t n_angles, 
 // `pow2`; `widen`: a block's widest direction against the mean.
 struct NodeCost {
   int gran = 64, tile = 512, from_zero = 1, pow2 = 0;
+  int64_t set_cut = -1;  // not chosen but asked for: so many energies, if they ascend
   float widen = 1.f, direct = 0.f, fixed = 0.f, per_run = 0.f, per_energy = 0.f, reach = 0.f, cap = 64.f;
   // for a kernel that fills only a part of the SMs (or lanes) the costs rise by that factor
   void scale(float f) {

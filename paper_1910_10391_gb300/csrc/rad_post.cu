@@ -63,6 +63,10 @@ __device__ void node_plan(const Params &P, const NodeCost &c_) {
   bad = __syncthreads_or(bad);
   const float windows = block_sum(cnt);
   if (bad || !(windows > 0.f)) return;
+  if (c_.set_cut >= 0) {
+    if (tid == 0) *P.node_cut = static_cast<int>(c_.set_cut);
+    return;
+  }
   const float step = widest * c_.widen;
   const float inv_E = P.mode == RAD_CLASSICAL ? 0.f : static_cast<float>(1.0 / P.energy[0]);
   auto ws = [&](int64_t i) {  // FP32: an estimate, and an FP64 division would cost 1000 clocks here
