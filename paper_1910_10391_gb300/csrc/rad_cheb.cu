@@ -80,6 +80,18 @@ __device__ __forceinline__ df2 to_df(double v) {
   return r;
 }
 
+// s + v, its rounding error added to e (Knuth's TwoSum); s - a b the same
+__device__ __forceinline__ void add_err(double &s, double &e, double v) {
+  const double t = s + v, b = t - s;
+  e += (s - (t - b)) + (v - b);
+  s = t;
+}
+__device__ __forceinline__ void sub_prod(double &s, double &e, double a, double b) {
+  const double p = __dmul_rn(a, b);
+  e -= fma(a, b, -p);
+  add_err(s, e, -p);
+}
+
 __device__ __forceinline__ void async16(void *dst, const void *src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
@@ -367,7 +379,12 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
           const int runs = (n + run - 1) / run;
           run = (n + runs - 1) / runs;
         }
-        const double A0 = ((cn * r0[F_T] - r0[F_DZ]) - nx * r0[F_X]) - ny * r0[F_Y];
+        // phase length of the window's reference, with its rounding error: all samples of a run share
+        // the run's base phase, so its error does not average out as that of a phase per sample does
+        double A0 = __dmul_rn(cn, r0[F_T]), A0e = fma(cn, r0[F_T], -A0);
+        add_err(A0, A0e, -r0[F_DZ]);
+        sub_prod(A0, A0e, nx, r0[F_X]);
+        sub_prod(A0, A0e, ny, r0[F_Y]);
         for (int k0 = 0; k0 < n; k0 += run) {
           const int m = n - k0 < run ? n - k0 : run;  // samples of this run
           auto length = [&](int k) {  // phase length from the window's reference
@@ -442,7 +459,8 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
           for (int i = 0; i < kM; ++i)
 #pragma unroll
             for (int c = 0; c < NP; ++c) Mv[i][c] = reinterpret_cast<const T *>(s_mom)[(i * NP + c) * 32 + lane];
-          const double Ac = A0 + ctr;
+          double Ac = A0, Ae = A0e;
+          add_err(Ac, Ae, ctr);
           // the next energy's coefficients and amplitudes are on their way from L2 while this one's
           // series is summed: eight warps an SM are too few to hide those loads
           unsigned char *ring = sm + SM::kRing + warp * 2 * SM::kSlot;
@@ -465,7 +483,7 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
           for (int e = warp; e < ne; e += kW, slot ^= 1) {
             fetch(e + kW, slot ^ 1);
             const int terms = terms_next;
-            const double phi = __dmul_rn(ws_next, Ac);
+            const double phi = __dmul_rn(ws_next, Ac), phi_e = fma(ws_next, Ae, fma(ws_next, Ac, -phi));
             if (e + kW < ne) {
               terms_next = n_terms[e + kW];
               ws_next = wsv[e + kW];
@@ -473,7 +491,10 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
             T sn, cs;
             float4 entry;
             float xh, xl;
-            if constexpr (DF) entry = tab[dfr::reduce_phase(phi, xh, xl) & (dfr::kTabN - 1)];
+            if constexpr (DF) {
+              entry = tab[dfr::reduce_phase(phi, xh, xl) & (dfr::kTabN - 1)];
+              xl = __fadd_rn(xl, __double2float_rn(phi_e));
+            }
             asm volatile("cp.async.wait_group 1;" ::: "memory");
             __syncwarp();
             const T *cf = reinterpret_cast<const T *>(ring + slot * SM::kSlot);
@@ -492,10 +513,13 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
                 }
               }
             }
-            if constexpr (DF)
+            if constexpr (DF) {
               dfr::sincos_from_entry(entry, xh, xl, sn.h, sn.l, cs.h, cs.l);
-            else
-              sincos_table(phi, P.table, sn, cs);
+            } else {
+              double r;
+              const int j = reduce_table(phi, r);
+              sincos_reduced(j, r + phi_e, P.table, sn, cs);
+            }
             A *o = amp + static_cast<size_t>(e) * 2 * NP * 32 + lane;
 #pragma unroll
             for (int c = 0; c < NP; ++c) {
