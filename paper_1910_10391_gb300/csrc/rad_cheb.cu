@@ -9,9 +9,9 @@
 //   sum_k f_k e^{i w a_k} = sum_m (2 - delta_m0) i^m J_m(w a_lim) M_m,  M_m = sum_k f_k T_m(x_k).
 // A sample then costs one recurrence step and one multiply-add per component and moment whatever
 // the number of energies, and an energy costs kM multiply-adds per component, one sin/cos of the
-// run's base phase and one rotation per run instead of per sample. With w_hi a_lim = 9 (5 for
-// spin 1/2, which has three components and keeps 24 moments instead of 32) the first dropped term is
-// below 1e-14; terms that are below 1e-18 at an energy's own w a_lim are left out for it.
+// run's base phase and one rotation per run instead of per sample. Spin 1/2 has three components and keeps 24
+// moments, the others 32; w_hi a_lim (Cheb::kPhi) keeps the first dropped term below the form's rounding;
+// terms that are below 1e-18 at an energy's own w a_lim are left out for it.
 //
 // Work split: a block of 4 warps takes 32 directions (one per lane: x_k, the recurrence and the
 // moments live in the lane's registers and need no exchange) and the energies of one tile. The warps
@@ -50,7 +50,12 @@ struct Cheb {
   static constexpr bool kSpin = MODE == RAD_SPIN_HALF;
   static constexpr int NP = kSpin ? 3 : 2;   // summed components (f_x, f_y, j)
   static constexpr int kM = kSpin ? 24 : 32;
-  static constexpr double kPhi = kSpin ? 5.0 : 9.0;
+  // Phase range w_hi a_lim. The samples of a run end at x = +-1, and where they add up coherently the tile's
+  // highest energies see the first dropped term, 2 J_kM(kPhi), at about a quarter: it is held to 1e-16
+  // of |f| in FP64 (at 5 and 9 it was 9e-15 and 4e-15: 4e-15 of the spectrum at the top of a tile), and below the
+  // float pairs' own 1e-14 in double-float.
+  template <bool DF>
+  static constexpr double kPhi = kSpin ? (DF ? 5.0 : 4.25) : (DF ? 9.0 : 8.25);
   static constexpr int kTile = kSpin ? 256 : 512;  // energies of a tile
 };
 
@@ -178,58 +183,51 @@ __device__ __forceinline__ double rcp_step(double v) {
 }
 
 // (2 - delta_m0) (-1)^{m/2} J_m(z) for m < M into out (as T), and the number of terms above 1e-18,
-// rounded up to even. Power series below z = 1/2 (ended where the terms pass 1e-18), Miller's backward
-// recurrence normalised by J_0 + 2 sum J_2k = 1 above (M. Abramowitz, I. A. Stegun, 9.12). One thread
-// per energy, once per energy tile and particle energy: an FP64 instruction costs the warp 64 clocks, so
-// there is no division in the loops.
+// rounded up to even. Power series below z = 2^-8 (its dropped terms are below 1e-18), Miller's backward
+// recurrence normalised by J_0 + 2 sum J_2k = 1 above (M. Abramowitz, I. A. Stegun, 9.12). All runs of an energy
+// share its coefficients, so their errors do not average out: 2/z and the normalising sum carry their
+// rounding errors (worst J_m over z 1.0 units of 2^-53, J_0 0.3 in the mean; 2.5 and 0.6 without). The unnormalised
+// values wait in out. One thread per energy, once per energy tile and particle energy: an FP64 instruction
+// costs the warp 64 clocks and the branches of a warp's lanes follow one another, so the recurrence has no division
+// and the series is a few instructions.
 template <bool DF, int M>
 __device__ int bessel_row(double z, typename Num<DF>::T *out) {
+  double *raw = reinterpret_cast<double *>(out);
   int terms = 2;
   auto put = [&](int m, double j) {
     const double v = (m ? 2.0 : 1.0) * ((m >> 1) & 1 ? -j : j);
     out[m] = Num<DF>::from(v);
     if (fabs(v) > 1e-18 && m + 1 > terms) terms = m + 1;
   };
-  if (z < 0.5) {
-    // J_m = (z/2)^m / m! sum_k q^k / (k! (m+1)..(m+k)), q = -z^2/4: with 1/((m+1)..(m+6)) over a common
-    // denominator the sum is one quotient
-    const double q = -0.25 * z * z;
-    double lead = 1.0;  // (z/2)^m / m!
-    for (int m = 0; m < M; ++m) {
-      double num = 0.0, den = 1.0;  // Horner from k = 6: 1 + q/(1 (m+1)) (1 + q/(2 (m+2)) (...))
-      for (int k = 6; k >= 1; --k) {
-        // (num, den) <- value 1 + q / (k (m + k)) * (num_k / den_k), kept as a fraction
-        const double inner = k == 6 ? 1.0 : num, id = k == 6 ? 1.0 : den, f = static_cast<double>(k * (m + k));
-        den = f * id;
-        num = fma(q, inner, den);
-      }
-      const double j = lead < 1e-19 ? 0.0 : lead * (num * rcp_step(den));
-      put(m, j);
-      lead *= 0.5 * z * rcp_step(m + 1.0);
-      if (lead < 1e-19) {
-        for (int i = m + 1; i < M; ++i) out[i] = Num<DF>::from(0.0);
-        break;
-      }
-    }
+  if (z < 0x1p-8) {
+    const double h = 0.5 * z, q = h * h;
+    put(0, fma(-q, fma(-q, fma(-q, 1.0 / 36.0, 0.25), 1.0), 1.0));
+    put(1, fma(-q, fma(-q, 1.0 / 12.0, 0.5), 1.0) * h);
+    put(2, fma(-q, fma(-q, 1.0 / 24.0, 1.0 / 3.0), 1.0) * (q * 0.5));
+    put(3, fma(-q, 0.25, 1.0) * (q * h * (1.0 / 6.0)));
+    put(4, q * q * (1.0 / 24.0));
+    put(5, q * q * h * (1.0 / 120.0));
+    for (int m = 6; m < M; ++m) out[m] = Num<DF>::from(0.0);  // below 1e-19
   } else {
-    const double rz = 2.0 / z;
-    // twice: the normalising sum first, then the values (no array of them)
-    constexpr int kStart = M + 24;
-    double hi = 0.0, lo = 1e-200, sum = 0.0;
-    for (int m = kStart; m > 0; --m) {
-      const double t = fma(m * rz, lo, -hi);  // J_{m-1}
+    const double rz = 2.0 / z, rl = fma(-rz, z, 2.0) / z;
+    double hi = 0.0, lo = 1e-200, sum = 0.0, err = 0.0;
+    double dm = M + 8;
+#pragma unroll 2
+    for (int m = M + 8; m > 0; --m, dm -= 1.0) {  // J_{M+8} is below 1e-21 for z <= 9
+      const double p = dm * rz, pe = fma(dm, rl, fma(dm, rz, -p));
+      const double t = fma(p, lo, fma(pe, lo, -hi));  // J_{m-1}
       hi = lo;
       lo = t;
-      if ((m - 1) % 2 == 0) sum += t;
+      if (m <= M) raw[m - 1] = t;
+      if (m % 2 != 0 && m > 1) add_err(sum, err, t);
     }
-    const double scale = 1.0 / (2.0 * sum - lo);
-    hi = 0.0;
-    lo = 1e-200;
-    for (int m = kStart; m > 0; --m) {
-      const double t = fma(m * rz, lo, -hi);
-      hi = lo;
-      lo = t;
-      if (m - 1 < M) put(m - 1, t * scale);
+    double norm = lo;
+    err *= 2.0;
+    add_err(norm, err, 2.0 * sum);
+    const double scale = 1.0 / norm, scale_e = (fma(-scale, norm, 1.0) - scale * err) * scale;
+    for (int m = 0; m < M; ++m) {
+      const double t = raw[m];
+      put(m, fma(t, scale, t * scale_e));
     }
   }
   return (terms + 1) & ~1;
@@ -310,7 +308,7 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
           const double w = __ddiv_rn(h, kHbarC);
           return MODE == RAD_CLASSICAL ? w : __ddiv_rn(w, __dsub_rn(1.0, __ddiv_rn(h, En)));
         };
-        a_lim = C::kPhi / ws_of(P.hw[e0 + ne - 1]);  // the energies ascend
+        a_lim = C::template kPhi<DF> / ws_of(P.hw[e0 + ne - 1]);  // the energies ascend
         __syncthreads();  // the last particle's series is no longer read
         for (int e = tid; e < ne; e += kW * 32) {
           const double w = ws_of(P.hw[e0 + e]);
@@ -637,7 +635,8 @@ NodeCost cheb_cost(int mode, bool df, int direct_gran) {
   c.tile = cheb_tile(mode);
   c.cap = kWin;
   c.widen = 1.6f;  // the widest of 32 directions, a row or more of a grid
-  c.reach = 0.95f * 2.f * static_cast<float>(spin ? Cheb<RAD_SPIN_HALF>::kPhi : Cheb<RAD_CLASSICAL>::kPhi);
+  c.reach = 0.95f * 2.f * static_cast<float>(spin ? (df ? Cheb<RAD_SPIN_HALF>::kPhi<true> : Cheb<RAD_SPIN_HALF>::kPhi<false>)
+                                                     : (df ? Cheb<RAD_CLASSICAL>::kPhi<true> : Cheb<RAD_CLASSICAL>::kPhi<false>));
   c.direct = df ? (spin ? 1.45f : 1.3f) : (spin ? 11.5f : 9.6f);
   c.fixed = df ? (spin ? 36.f : 32.f) : 85.f;
   c.per_run = df ? 20.f : 110.f;
