@@ -44,6 +44,11 @@ namespace {
 constexpr int kW = 4;        // warps per block
 constexpr int kWin = 256;    // samples of a window, the longest run
 constexpr int kRecW = 10;    // doubles per prepared sample
+// A particle's amplitudes are added up over kFlush runs at a time and these sums in FP64: the rounding of each
+// addition grows with the sum that it is added to (in one float-pair sum over the 2000 runs of 12000
+// samples the spectrum was off by 1.1e-12, in FP64 by 1.1e-15; 2e-14 and 8e-16 by the direct kernels).
+template <bool DF>
+constexpr int kFlush = DF ? 64 : 16;
 
 template <int MODE>
 struct Cheb {
@@ -115,6 +120,7 @@ struct Num<false> {
   static __device__ __forceinline__ void mac(A &a, T x, T y) { a = fma(x, y, a); }
   static __device__ __forceinline__ void add(A &a, T x) { a += x; }
   static __device__ __forceinline__ T value(A a) { return a; }
+  static __device__ __forceinline__ A settle(A a) { return a; }
   static __device__ __forceinline__ double to_double(A a) { return a; }
 };
 template <>
@@ -137,22 +143,26 @@ struct Num<true> {
     dfr::two_sum(a.h, a.l, s, t);
     return {s, t};
   }
+  // the sum with its errors moved into the leading part: left beside it they are rounded at their own, growing size
+  static __device__ __forceinline__ A settle(const A &a) { return value(a); }
   static __device__ __forceinline__ double to_double(const A &a) {
     return static_cast<double>(a.h) + static_cast<double>(a.l);
   }
 };
 
-// A block's scratch for n energies (the tile, or all of the call's if fewer): amplitudes [n][2 NP][32],
+// A block's scratch for n energies (the tile, or all of the call's if fewer): amplitudes of the last runs and
+// of those before [n][2 NP][32] each,
 // particle sums S [n][32], series coefficients [n][kM], w* [n], number of terms [n] and (DF) the
 // float-pair sin/cos table; every part on 16 bytes.
 template <int MODE>
 struct Scratch {
   using C = Cheb<MODE>;
-  size_t amp, s, coef, ws, terms, tab, total;
+  size_t amp, sum, s, coef, ws, terms, tab, total;
   __host__ __device__ explicit Scratch(int64_t n_omega) {
     const size_t n = (static_cast<size_t>(n_omega < C::kTile ? n_omega : C::kTile) + 3) / 4 * 4;
     amp = 0;
-    s = amp + n * 2 * C::NP * 32 * 8;
+    sum = amp + n * 2 * C::NP * 32 * 8;
+    s = sum + n * 2 * C::NP * 32 * 8;
     coef = s + n * 32 * 8;
     ws = coef + n * C::kM * 8;
     terms = ws + n * 8;
@@ -171,7 +181,11 @@ struct Smem {
   static constexpr int kSlot = C::kM * 8 + 2 * C::NP * 32 * 8;
   static constexpr int kRing = kStep + kWin * 16;
   static constexpr int kMisc = kRing + kW * 2 * kSlot;               // item, status; float [4]
-  static constexpr int kTotal = kMisc + 64;
+  // double [4][32]: each lane's phase length and its error at the run's centre and at the window's reference, the same
+  // in the four warps (which write the same values, behind the barriers that end the last run's reads); two blocks
+  // fit an SM with 1 KB of it, not with 4
+  static constexpr int kBase = kMisc + 64;
+  static constexpr int kTotal = kBase + 4 * 32 * 8;
 };
 
 // 1 / v for normal v: one cubic step from the hardware's 20-bit reciprocal
@@ -248,6 +262,7 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
   A *s_mom = reinterpret_cast<A *>(sm + SM::kMom);
   float4 *s_step = reinterpret_cast<float4 *>(sm + SM::kStep);
   int *s_item = reinterpret_cast<int *>(sm + SM::kMisc);
+  volatile double *s_base = reinterpret_cast<volatile double *>(sm + SM::kBase);
   float *s_max = reinterpret_cast<float *>(s_item + 2);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
@@ -320,7 +335,9 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
       const double inv_a = 1.0 / a_lim;
       const double cns = cn * inv_a, nxs = nx * inv_a, nys = ny * inv_a;
       const float cnf = static_cast<float>(cn), nxf = static_cast<float>(nx), nyf = static_cast<float>(ny);
-      bool first = true;  // first run of the particle's piece: amplitudes are written, not added to
+      // runs since the last flush, plus 256 once there was one (one register); the first run of a
+      // particle's piece or after a flush writes its amplitudes, the others add to them
+      int since = 0;
       for (int64_t w0 = kb; w0 < ke; w0 += kWin) {
         const int n = static_cast<int>(ke - w0 < kWin ? ke - w0 : kWin);
         const double *r0 = S + w0 * kRec;  // the window's reference
@@ -383,6 +400,8 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
         add_err(A0, A0e, -r0[F_DZ]);
         sub_prod(A0, A0e, nx, r0[F_X]);
         sub_prod(A0, A0e, ny, r0[F_Y]);
+        s_base[64 + lane] = A0;  // registers are what is short here
+        s_base[96 + lane] = A0e;
         for (int k0 = 0; k0 < n; k0 += run) {
           const int m = n - k0 < run ? n - k0 : run;  // samples of this run
           auto length = [&](int k) {  // phase length from the window's reference
@@ -457,8 +476,12 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
           for (int i = 0; i < kM; ++i)
 #pragma unroll
             for (int c = 0; c < NP; ++c) Mv[i][c] = reinterpret_cast<const T *>(s_mom)[(i * NP + c) * 32 + lane];
-          double Ac = A0, Ae = A0e;
-          add_err(Ac, Ae, ctr);
+          {
+            double Ac = s_base[64 + lane], Ae = s_base[96 + lane];
+            add_err(Ac, Ae, ctr);
+            s_base[lane] = Ac;
+            s_base[32 + lane] = Ae;
+          }
           // the next energy's coefficients and amplitudes are on their way from L2 while this one's
           // series is summed: eight warps an SM are too few to hide those loads
           unsigned char *ring = sm + SM::kRing + warp * 2 * SM::kSlot;
@@ -467,7 +490,7 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
               unsigned char *d = ring + slot * SM::kSlot;
               const unsigned char *c = reinterpret_cast<const unsigned char *>(coef + static_cast<size_t>(e) * kM);
               if (lane < kM / 2) async16(d + lane * 16, c + lane * 16);
-              if (!first) {
+              if (since & 255) {
                 const unsigned char *a = reinterpret_cast<const unsigned char *>(amp + static_cast<size_t>(e) * 2 * NP * 32);
 #pragma unroll
                 for (int i = 0; i < NP; ++i) async16(d + kM * 8 + (i * 32 + lane) * 16, a + (i * 32 + lane) * 16);
@@ -481,7 +504,8 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
           for (int e = warp; e < ne; e += kW, slot ^= 1) {
             fetch(e + kW, slot ^ 1);
             const int terms = terms_next;
-            const double phi = __dmul_rn(ws_next, Ac), phi_e = fma(ws_next, Ae, fma(ws_next, Ac, -phi));
+            const double Ac = s_base[lane], phi = __dmul_rn(ws_next, Ac);
+            const double phi_e = fma(ws_next, s_base[32 + lane], fma(ws_next, Ac, -phi));
             if (e + kW < ne) {
               terms_next = n_terms[e + kW];
               ws_next = wsv[e + kW];
@@ -521,18 +545,27 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
             A *o = amp + static_cast<size_t>(e) * 2 * NP * 32 + lane;
 #pragma unroll
             for (int c = 0; c < NP; ++c) {
-              A zr = first ? N::zero() : old[(2 * c) * 32], zi = first ? N::zero() : old[(2 * c + 1) * 32];
+              A zr = since & 255 ? old[(2 * c) * 32] : N::zero(), zi = since & 255 ? old[(2 * c + 1) * 32] : N::zero();
               const T vr = N::value(re[c]), vi = N::value(im[c]);
               N::mac(zr, cs, vr);
               N::mac(zr, N::neg(sn), vi);
               N::mac(zi, sn, vr);
               N::mac(zi, cs, vi);
-              o[(2 * c) * 32] = zr;
-              o[(2 * c + 1) * 32] = zi;
+              o[(2 * c) * 32] = N::settle(zr);
+              o[(2 * c + 1) * 32] = N::settle(zi);
             }
             __syncwarp();  // the slot is read; the fetch after next refills it
           }
-          first = false;
+          if ((++since & 255) == kFlush<DF>) {  // each lane its own amplitudes
+            double *total = reinterpret_cast<double *>(amp + sc.sum / 8);
+            for (int e = warp; e < ne; e += kW) {
+              const size_t at = static_cast<size_t>(e) * 2 * NP * 32 + lane;
+#pragma unroll 1
+              for (int c = 0; c < 2 * NP; ++c)
+                total[at + c * 32] = N::to_double(amp[at + c * 32]) + (since & 256 ? total[at + c * 32] : 0.0);
+            }
+            since = 256;
+          }
         }
       }
       // the particle's (piece's) amplitudes: each warp its own energies
@@ -540,7 +573,8 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
         double a[2 * NP];
 #pragma unroll
         for (int c = 0; c < 2 * NP; ++c)
-          a[c] = first ? 0.0 : N::to_double(amp[(static_cast<size_t>(e) * 2 * NP + c) * 32 + lane]);
+          a[c] = (since & 255 ? N::to_double(amp[(static_cast<size_t>(e) * 2 * NP + c) * 32 + lane]) : 0.0) +
+                 (since & 256 ? reinterpret_cast<double *>(amp + sc.sum / 8)[(static_cast<size_t>(e) * 2 * NP + c) * 32 + lane] : 0.0);
         if (P.amp_mode) {
           if (jdir < P.n_angles) {
 #pragma unroll
