@@ -43,16 +43,19 @@ constexpr float kXiMax = 1.57079632679489662f;  // |h a_k| at twofold oversampli
 
 // The Kaiser-Bessel window I0(beta sqrt(1 - (2u/8)^2)), beta = 18.661, over its Fourier transform at
 // 0, on the four unit intervals u in [3,4], [2,3], [1,2], [0,1] as polynomials in z = 2 frac(u) - 1
-// (Chebyshev fits, error below 1e-9); the other four intervals mirror them.
+// (Chebyshev fits, error below 1e-9); the other four intervals mirror them. All of it times 1 + 1.65e-7: the
+// SFU's sin and cos are short of modulus 1 by 1.0e-7 in the mean, and this form multiplies three of them (node,
+// centre frequency and run) where the direct kernel has two, so that its peaks came out 4.7e-7 too
+// low (2.1e-7 directly; means over bins above 5 % of the peak).
 __constant__ float kKbRow[4][9] = {
-    {4.143404153e-05f, -1.647157490e-04f, 2.796029959e-04f, -2.649951424e-04f, 1.526979771e-04f, -5.340337630e-05f,
-     9.562848215e-06f, 3.008195447e-07f, -4.480139766e-07f},
-    {8.204613101e-03f, -1.478727248e-02f, 1.093403570e-02f, -3.991892863e-03f, 5.446627406e-04f, 1.068984792e-04f,
-     -4.987233109e-05f, 3.268000232e-06f, 1.223624974e-06f},
-    {1.155014882e-01f, -1.057883315e-01f, 2.801810393e-02f, 2.838173613e-03f, -2.546929184e-03f, 2.065807465e-04f,
-     9.103259867e-05f, -1.478784324e-05f, -1.669980253e-06f},
-    {3.762524844e-01f, -1.075457502e-01f, -3.923190424e-02f, 1.330029539e-02f, 1.849859379e-03f, -7.821834401e-04f,
-     -5.083792701e-05f, 2.760262528e-05f, 8.255164980e-07f}};
+    {4.143404837e-05f, -1.647157762e-04f, 2.796030420e-04f, -2.649951861e-04f, 1.526980023e-04f, -5.340338511e-05f,
+     9.562849793e-06f, 3.008195943e-07f, -4.480140505e-07f},
+    {8.204614455e-03f, -1.478727492e-02f, 1.093403750e-02f, -3.991893522e-03f, 5.446628305e-04f, 1.068984968e-04f,
+     -4.987233932e-05f, 3.268000771e-06f, 1.223625176e-06f},
+    {1.155015073e-01f, -1.057883490e-01f, 2.801810855e-02f, 2.838174081e-03f, -2.546929604e-03f, 2.065807806e-04f,
+     9.103261369e-05f, -1.478784568e-05f, -1.669980529e-06f},
+    {3.762525465e-01f, -1.075457679e-01f, -3.923191071e-02f, 1.330029758e-02f, 1.849859684e-03f, -7.821835692e-04f,
+     -5.083793540e-05f, 2.760262983e-05f, 8.255166342e-07f}};
 
 __device__ __forceinline__ float kb_row(int row, float z) {
   float v = kKbRow[row][8];

@@ -73,7 +73,7 @@ def errors(got, ref):
     return np.linalg.norm(e) / np.linalg.norm(ref), np.median(e / np.maximum(ref, 1e-6 * ref.max()))
 
 
-@pytest.mark.parametrize("form", [rad.RAD_FP64, rad.RAD_FP64_DF])
+@pytest.mark.parametrize("form", [rad.RAD_FP64, rad.RAD_FP64_DF, rad.RAD_MIXED])
 @pytest.mark.parametrize("kind,mode", [("undulator", rad.RAD_CLASSICAL), ("positrons", rad.RAD_CLASSICAL),
                                        ("positrons", rad.RAD_SPIN_HALF), ("top", rad.RAD_CLASSICAL),
                                        ("top", rad.RAD_SPIN_HALF)])
@@ -91,12 +91,12 @@ def test_no_further_from_the_exact_sum_than_directly(form, kind, mode):
     assert all(r <= max(1.1 * d, 4.4e-16) for r, d in zip(err[inp.n_omega], err[0])), err
 
 
-@pytest.mark.parametrize("form", [rad.RAD_FP64, rad.RAD_FP64_DF])
+@pytest.mark.parametrize("form", [rad.RAD_FP64, rad.RAD_FP64_DF, rad.RAD_MIXED])
 def test_long_trajectory_in_one_piece(form):
     """Per-particle spectra keep a trajectory in one piece, so that its amplitudes collect some hundred runs."""
     import torch
     tr = I.channeling(2, 10e9, +1, 12000, 5e-9, 3)
-    grid = I.Grid(I.omega_log(64, 1e7, 1e9), *directions(16))
+    grid = I.Grid(I.omega_log(96 if form == rad.RAD_MIXED else 64, 1e7, 1e9), *directions(16))
     ref = exact_cube(tr, grid, rad.RAD_SPIN_HALF)
     inp = rad.DeviceInputs(tr, grid)
     p, _ = plan_of(inp, rad.RAD_SPIN_HALF, form, rad.RAD_PER_PARTICLE | 2)
