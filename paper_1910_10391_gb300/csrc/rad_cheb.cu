@@ -188,14 +188,6 @@ struct Smem {
   static constexpr int kTotal = kBase + 4 * 32 * 8;
 };
 
-// 1 / v for normal v: one cubic step from the hardware's 20-bit reciprocal
-__device__ __forceinline__ double rcp_step(double v) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
-  const double e = fma(-v, r, 1.0);
-  return fma(fma(e, e, e), r, r);
-}
-
 // (2 - delta_m0) (-1)^{m/2} J_m(z) for m < M into out (as T), and the number of terms above 1e-18,
 // rounded up to even. Power series below z = 2^-8 (its dropped terms are below 1e-18), Miller's backward
 // recurrence normalised by J_0 + 2 sum J_2k = 1 above (M. Abramowitz, I. A. Stegun, 9.12). All runs of an energy
@@ -422,7 +414,7 @@ __global__ void __launch_bounds__(kW * 32, 2) k_cheb(const Params P, unsigned ch
             const double x = fma(-nys, o[3], fma(-nxs, o[2], fma(-inv_a, o[1], fma(cns, o[0], off_x))));
             const double vx = o[4], vy = o[5];
             const double D = cn - o[9] - nx * vx - ny * vy;  // 1 - n.beta (Sec. II, g)
-            const double r = rcp_step(D), g = r * r;
+            const double r = __drcp_rn(D), g = r * r;
             const double a = nx - vx, b = ny - vy;
             const double mm = fma(ny, o[7], fma(nx, o[6], o[8]));  // n.beta_dot, weighted
             T f[NP];

@@ -385,29 +385,6 @@ __device__ __forceinline__ State deriv_axial(const Chan &C, const Axial &A, doub
 // Pieces of the tabulated and of the lane-group kernels: FP64 divisions and square roots cost some
 // ten dependent instructions each, and a step is one dependent chain.
 // ------------------------------------------------------------------------------------
-// 1 / v for normal v: one cubic step from the hardware's 20-bit reciprocal
-__device__ __forceinline__ double rcp_fast(double v) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
-  const double e = fma(-v, r, 1.0);
-  return fma(fma(e, e, e), r, r);
-}
-
-// sqrt(a) and 1 / sqrt(a), 0 and infinity where 0 <= a < 1e-300 and NaN below: one cubic step from the
-// hardware's reciprocal root and a Newton correction of the root. No branch: the chains around it
-// interleave.
-__device__ __forceinline__ double sqrt_fast(double a, double &inv) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-  const double e = fma(-(a * y), y, 1.0);
-  const double z = fma(y * e, fma(e, 0.375, 0.5), y);
-  const bool zero = a >= 0.0 && a < 1e-300;
-  inv = zero ? INFINITY : z;
-  const double r = a * z;
-  const double root = fma(0.5 * z, fma(-r, r, a), r);
-  return zero ? 0.0 : root;
-}
-
 // What a stage needs of the energy: g, 1/E, 1/g^2 and the energy part of the longitudinal velocity
 // (1/g0^2 - 1/g^2 and 1 - 1/g^2)
 struct EnergyPart {
@@ -416,7 +393,7 @@ struct EnergyPart {
 __device__ __forceinline__ EnergyPart energy_part(double E, double inv_mass, double g0, double ig02) {
   EnergyPart e;
   e.g = E * inv_mass;
-  const double ig = rcp_fast(e.g);
+  const double ig = __drcp_rn(e.g);
   e.inv_E = ig * inv_mass;
   e.ig2 = ig * ig;
   e.d_inv = ((e.g - g0) * (e.g + g0)) * (e.ig2 * ig02);
@@ -426,8 +403,9 @@ __device__ __forceinline__ EnergyPart energy_part(double E, double inv_mass, dou
 
 // v_z - beta0 (see dvz_of) and 1 / v_z
 __device__ __forceinline__ double dvz_fast(const EnergyPart &e, double q0, double beta0, double vp2, double &inv_vz) {
-  const double vz = sqrt_fast(e.one - vp2, inv_vz);
-  return (e.d_inv - vp2 - q0) * rcp_fast(vz + beta0);
+  const double vz = sqrt(e.one - vp2);
+  inv_vz = __drcp_rn(vz);
+  return (e.d_inv - vp2 - q0) * __drcp_rn(vz + beta0);
 }
 
 // Electron part of the scattering variance per (1/2) dt pi r0^2 n_el. The logarithm of q = 2 m_e/I
@@ -454,7 +432,7 @@ struct Bracket {
     t = fma(d, t, 1.0 / 3.0);
     t = fma(d, t, -1.0 / 2.0);
     const double br = fmax(fma(d * d, t, d) + log_ref - e.one, 0.0);
-    return br * e.ig2 * rcp_fast(e.one * e.one);
+    return br * e.ig2 * __drcp_rn(e.one * e.one);
   }
 };
 
@@ -499,7 +477,7 @@ __device__ __forceinline__ void axis_sums_fast(double u0, double L, int K, doubl
     s0 += E;
   }
   E = E0;
-  rho = q * rcp_fast(up);
+  rho = q * __drcp_rn(up);
   u = r;
   for (int m = 0; m < K + i0; ++m) {  // images i0 - 1 .. -K at r + m L
     E *= rho;
@@ -724,8 +702,7 @@ __global__ void k_axial_group(const Chan C, const Axial A, int64_t n_particles, 
         if (lane_k == 0) kick_normals(seed, pid, static_cast<uint64_t>(k + gl), z0, z1);
         double var = C.var_k * (ep.inv_E * ep.inv_E) * n_nuc;
         if (A.el) var = fma(n_el, bk.value(A.lk, ep), var);
-        double inv_sd;
-        const double sd = sqrt_fast(var, inv_sd);
+        const double sd = sqrt(var);
         const double dthx = sd * __shfl_sync(mask, z0, lane_k, W), dthy = sd * __shfl_sync(mask, z1, lane_k, W);
         kx = dthx * inv_dt;
         ky = dthy * inv_dt;
@@ -860,7 +837,7 @@ __global__ void __launch_bounds__(kTabThreads) k_channel_tab(
     const double g0 = E0 * inv_mass, ig02 = 1.0 / (g0 * g0);
     const double beta0 = 1.0 - 0.5 * ig02, q0 = 0.25 * (ig02 * ig02);
     double x = x0[p], y = 0.0, vx = thx0[p], vy = thy0 ? thy0[p] : 0.0, dz = 0.0, E = E0;
-    double g = E * inv_mass, ig = rcp_fast(g);
+    double g = E * inv_mass, ig = __drcp_rn(g);
     Bracket bk{0.0, 0.0};  // 0 q - 1 is out of range: the first use sets the reference
     double kx = 0.0, ky = 0.0, z0 = 0.0, z1 = 0.0;
     double F = tab_eval(scale, tab, x);
@@ -880,7 +857,7 @@ __global__ void __launch_bounds__(kTabThreads) k_channel_tab(
           const double h = i < 3 ? hh : dt;
           if (C.ll) {
             gs[i] = fma(h, dEs[i - 1], E) * inv_mass;
-            igs[i] = rcp_fast(gs[i]);
+            igs[i] = __drcp_rn(gs[i]);
           }
           vs[i] = fma(h, as[i - 1], vx);
           drive(i, tab_eval(scale, tab, fma(h, vs[i - 1], x)));
@@ -941,7 +918,7 @@ __global__ void __launch_bounds__(kTabThreads) k_channel_tab(
       if (C.ll) {
         E += h6 * (dEs[0] + 2.0 * dEs[1] + 2.0 * dEs[2] + dEs[3]);
         g = E * inv_mass;
-        ig = rcp_fast(g);
+        ig = __drcp_rn(g);
       }
       // the force at the next record's position, and the densities of the kick there
       const double own = tab_eval(scale, mine, x);
@@ -955,8 +932,7 @@ __global__ void __launch_bounds__(kTabThreads) k_channel_tab(
           const EnergyPart e{g, 0.0, i2, 0.0, 1.0 - i2};
           var = fma(G == 1 ? tab_eval(scale, tab + 2 * kTabI * kTabC, x) : from(own, 2), bk.value(P.lk, e), var);
         }
-        double inv_sd;
-        const double sd = sqrt_fast(var, inv_sd);
+        const double sd = sqrt(var);
         const double dthx = sd * from(z0, lane_k), dthy = sd * from(z1, lane_k);
         kx = dthx * inv_dt;
         ky = dthy * inv_dt;
@@ -965,7 +941,7 @@ __global__ void __launch_bounds__(kTabThreads) k_channel_tab(
         if (C.ms_loss) {
           E -= C.loss_k * (g * g * g) * (dthx * dthx + dthy * dthy);
           g = E * inv_mass;
-          ig = rcp_fast(g);
+          ig = __drcp_rn(g);
         }
       }
     }
