@@ -718,26 +718,27 @@ __global__ void k_axial_group(const Chan C, const Axial A, int64_t n_particles, 
 }
 
 // ------------------------------------------------------------------------------------
-// Doyle-Turner planar potential from a table. Force and densities are functions of the position
+// Doyle-Turner planar potential from a table. Force and electron density are functions of the position
 // within one cell [0, d_p) only, so every block expands them once, at the centres of kTabI equal
 // intervals, in Taylor polynomials of degree kTabDeg (Gaussians: g = e^{-k (r + s)^2} has
 // (n+1) g_{n+1} = -2 k r g_n - 2 k g_{n-1}), and a stage costs one polynomial instead of three
 // exponentials per term of the fit. With intervals of at most a tenth of the narrowest Gaussian's
 // sqrt(C) (tab_fits) the first dropped term is below 1e-16 of that Gaussian. The table takes about
-// 0.2 ms a block. 1024 particles x 2000 steps with every part of the physics: 75.0 ms by direct sums on
-// 8 lanes, 16.9 ms.
+// 0.2 ms a block. The nuclear density is not in it: it falls by e^{-160} between two planes, and the kicks of a particle
+// that stays there follow it, while a table's error is a fraction of the peak. 1024 particles x 2000 steps with
+// every part of the physics: 75.0 ms by direct sums on 8 lanes, 20.0 ms.
 //
 // An FP64 instruction occupies an SM sub-partition for 64 clocks whatever its active lanes, so the time
 // of a step is the number of FP64 instructions of a warp. G = 8 lanes hold one particle as long as the
-// warps, four particles each, have sub-partitions of their own (kTabGroupBelow = 4 x 608): lanes 0 to 2
-// evaluate force, nuclear and electron density at once, lanes 0 to 3 one RK4 stage's longitudinal
+// warps, four particles each, have sub-partitions of their own (kTabGroupBelow = 4 x 608): lanes 0
+// and 1 evaluate force and electron density and the nuclear density of one plane each at once, lanes 0 to 3 one RK4 stage's longitudinal
 // velocity each, every lane draws the kicks of one of the next eight steps, and the lanes share the
 // record's stores. G = 1 beyond.
 // ------------------------------------------------------------------------------------
 constexpr int kTabI = 256, kTabDeg = 11, kTabC = kTabDeg + 1;
 constexpr int kTabThreads = 128;
 constexpr int64_t kTabGroupBelow = 2432;
-constexpr size_t kTabBytes = sizeof(double) * 3 * kTabI * kTabC;
+constexpr size_t kTabBytes = sizeof(double) * 2 * kTabI * kTabC;
 
 // The polynomials resolve the fit: intervals of at most a tenth of the narrowest Gaussian.
 inline bool tab_fits(const Planar &P, const Chan &C) {
@@ -765,22 +766,19 @@ __device__ __forceinline__ void tab_add(double (&c)[kTabC], double amp, double k
   }
 }
 
-// table: 0 force, 1 n(x)/N, 2 (1/2) dt pi r0^2 n_el
+// table: 0 force, 1 the X-ray Gaussians' part of (1/2) dt pi r0^2 n_el
 __device__ void tab_build(const Chan &C, const Planar &P, double *tab) {
   const double h = C.d_p / kTabI;  // powers of the offset in intervals, |s| <= 1/2
-  const int n_tab = C.ms ? (P.el ? 3 : 2) : 1;
+  const int n_tab = C.ms && P.el ? 2 : 1;
   for (int u = threadIdx.x; u < n_tab * kTabI; u += kTabThreads) {
     const int t = u / kTabI, i = u - t * kTabI;
     const double x = (i + 0.5) * h;
     double c[kTabC];
 #pragma unroll
     for (int n = 0; n < kTabC; ++n) c[n] = 0.0;
-    if (t != 0)  // nuclear density: the two nearest planes
-      for (int j = 0; j < 2; ++j) tab_add(c, t == 1 ? C.dens_pref : P.ecx * C.dens_pref, C.inv_rho2, x - j * C.d_p, h, false);
-    if (t != 1)
-      for (int j = 1 - P.K; j <= P.K; ++j)
-        for (int m = 0; m < P.nt; ++m)
-          tab_add(c, t ? P.ek[m] : P.fk[m], t ? P.eck[m] : P.ck[m], x - j * C.d_p, h, t == 0);
+    for (int j = 1 - P.K; j <= P.K; ++j)
+      for (int m = 0; m < P.nt; ++m)
+        tab_add(c, t ? P.ek[m] : P.fk[m], t ? P.eck[m] : P.ck[m], x - j * C.d_p, h, t == 0);
 #pragma unroll
     for (int n = 0; n < kTabC; ++n) tab[u * kTabC + n] = c[n];
   }
@@ -822,7 +820,7 @@ __global__ void __launch_bounds__(kTabThreads) k_channel_tab(
   const unsigned mask = G == 1 ? 1u << (threadIdx.x & 31) : 0xFFu << (threadIdx.x & 24);
   const double inv_mass = 1.0 / C.mass, inv_dt = 1.0 / dt, h6 = dt / 6.0, hh = 0.5 * dt, scale = C.inv_d * kTabI;
   // this lane's table in the joint evaluation
-  const double *mine = tab + ((gl == 1 && C.ms) ? kTabI * kTabC : (gl == 2 && P.el) ? 2 * kTabI * kTabC : 0);
+  const double *mine = tab + (gl == 1 && C.ms && P.el ? kTabI * kTabC : 0);
   auto from = [&](double v, int l) { return G == 1 ? v : __shfl_sync(mask, v, l, G); };
   const int64_t stride = static_cast<int64_t>(gridDim.x) * (kTabThreads / G);
   for (int64_t p = blockIdx.x + static_cast<int64_t>(threadIdx.x / G) * gridDim.x; p < n_particles; p += stride) {
@@ -927,10 +925,19 @@ __global__ void __launch_bounds__(kTabThreads) k_channel_tab(
         const int lane_k = static_cast<int>(k % G);
         if (lane_k == 0) kick_normals(seed, pid, static_cast<uint64_t>(k + gl), z0, z1);
         const double i2 = ig * ig;
-        double var = C.var_k * (i2 * (inv_mass * inv_mass)) * (G == 1 ? tab_eval(scale, tab + kTabI * kTabC, x) : from(own, 1));
+        double n_nuc;
+        if (G == 1) {
+          n_nuc = plane_density(C, x);
+        } else {  // plane_density with one of the two planes per lane
+          const double m = floor(x * C.inv_d), r = (gl & 1) ? (m + 1.0) * C.d_p - x : x - m * C.d_p;
+          const double one = exp(-(r * r) * C.inv_rho2);
+          n_nuc = C.dens_pref * (from(one, 0) + from(one, 1));
+        }
+        double var = C.var_k * (i2 * (inv_mass * inv_mass)) * n_nuc;
         if (P.el) {
           const EnergyPart e{g, 0.0, i2, 0.0, 1.0 - i2};
-          var = fma(G == 1 ? tab_eval(scale, tab + 2 * kTabI * kTabC, x) : from(own, 2), bk.value(P.lk, e), var);
+          const double n_el = fma(P.ecx, n_nuc, G == 1 ? tab_eval(scale, tab + kTabI * kTabC, x) : from(own, 1));
+          var = fma(n_el, bk.value(P.lk, e), var);
         }
         const double sd = sqrt(var);
         const double dthx = sd * from(z0, lane_k), dthy = sd * from(z1, lane_k);
