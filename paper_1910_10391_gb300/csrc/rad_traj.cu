@@ -722,8 +722,7 @@ __global__ void k_axial_group(const Chan C, const Axial A, int64_t n_particles, 
 // within one cell [0, d_p) only, so every block expands them once, at the centres of kTabI equal
 // intervals, in Taylor polynomials of degree kTabDeg (Gaussians: g = e^{-k (r + s)^2} has
 // (n+1) g_{n+1} = -2 k r g_n - 2 k g_{n-1}), and a stage costs one polynomial instead of three
-// exponentials per term of the fit. With intervals of at most a tenth of the narrowest Gaussian's
-// sqrt(C) (tab_fits) the first dropped term is below 1e-16 of that Gaussian. The table takes about
+// exponentials per term of the fit. tab_fits says which fits the polynomials resolve. The table takes about
 // 0.2 ms a block. The nuclear density is not in it: it falls by e^{-160} between two planes, and the kicks of a particle
 // that stays there follow it, while a table's error is a fraction of the peak. 1024 particles x 2000 steps with
 // every part of the physics: 75.0 ms by direct sums on 8 lanes, 20.0 ms.
@@ -740,15 +739,25 @@ constexpr int kTabThreads = 128;
 constexpr int64_t kTabGroupBelow = 2432;
 constexpr size_t kTabBytes = sizeof(double) * 2 * kTabI * kTabC;
 
-// The polynomials resolve the fit: intervals of at most a tenth of the narrowest Gaussian.
+// The polynomials resolve the fit. A Gaussian of e^{-k r^2} leaves out, at half an interval of h = d_p / kTabI, at most
+// max |H_13(u) e^{-u^2}| / (2 12!) (h sqrt(k) / 2)^12 = 7.8e-3 (h sqrt(k) / 2)^12 of its force in units of the largest force's
+// 0.43 / sqrt(k), 2^-53 of it at h^2 k = 0.0197 (the density less); that is the bound for the narrowest term. Away from its
+// plane the error is (2 k r h / 2)^12 / 12! of the Gaussian itself, 1e-16 in the middle between two planes at k d_p^2 =
+// 125: the widest term of the force and that of the electron density, which make up the sums there, have to be below that.
+// Fits beyond either bound take the direct sums (128-thread blocks or lane groups: 75.2 ms where the table takes 20.0).
 inline bool tab_fits(const Planar &P, const Chan &C) {
   const double h = C.d_p / kTabI;
-  double k = C.ms ? C.inv_rho2 : 0.0;
+  double most = 0.0, least = INFINITY, least_el = INFINITY;
   for (int i = 0; i < P.nt; ++i) {
-    k = fmax(k, P.ck[i]);
-    if (P.el) k = fmax(k, P.eck[i]);
+    most = fmax(most, P.ck[i]);
+    least = fmin(least, P.ck[i]);
+    if (P.el) {
+      most = fmax(most, P.eck[i]);
+      least_el = fmin(least_el, P.eck[i]);
+    }
   }
-  return h * h * k <= 0.0101;
+  if (P.el) least = fmax(least, least_el);
+  return h * h * most <= 0.0197 && C.d_p * C.d_p * least <= 125.0;
 }
 
 __device__ __forceinline__ void tab_add(double (&c)[kTabC], double amp, double k, double r, double h, bool times_r) {
