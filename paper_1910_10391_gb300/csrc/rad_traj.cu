@@ -28,6 +28,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "rad_internal.cuh"
 
 namespace rad {
@@ -436,6 +438,14 @@ struct Bracket {
   }
 };
 
+// SM sub-partitions of the current device, four per SM: as many warps run without sharing an issue port
+int64_t sub_partitions() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    (void)cudaGetLastError();
+  return 4 * static_cast<int64_t>(std::max(sms, 1));
+}
+
 // Small ensembles: one particle per group of kGroup lanes. The lanes share the force evaluation
 // (each takes some of the (basis string, term) pairs, the partial forces are summed by a butterfly
 // of shuffles within the group) and keep identical copies of the state, so a step's exponentials
@@ -599,12 +609,11 @@ __device__ __forceinline__ AxialStage axial_stage(const Chan &C, const EnergyPar
 // The record's force is the first stage's, so a step evaluates the force four times; the divisions
 // and roots of the kinematics are the short forms above, and every lane draws the kick of one of the
 // next W steps. W = 32 lanes per particle as long as every warp has an SM sub-partition of its own
-// (kWarpBelow): an FP64 instruction occupies the sub-partition for 64 clocks whatever its active lanes,
+// (sub_partitions): an FP64 instruction occupies the sub-partition for 64 clocks whatever its active lanes,
 // so the time of a step is the number of FP64 instructions of a warp. 512 particles x 1000 steps of the
 // <110> axis: 73.6 ms with 128-thread blocks, five force sums a step and IEEE divisions; 35.7 ms with
 // these taken out, on 16 lanes; 23.1 ms on 32. (Tried and slower: branch-free exponentials and masked
 // image loops, 38.2 against 35.7 ms.)
-constexpr int64_t kWarpBelow = 609;
 template <int W>
 __global__ void k_axial_group(const Chan C, const Axial A, int64_t n_particles, const int64_t *__restrict__ offsets,
                               int64_t n_total, const double *__restrict__ energy, const double *__restrict__ x0,
@@ -729,14 +738,13 @@ __global__ void k_axial_group(const Chan C, const Axial A, int64_t n_particles, 
 //
 // An FP64 instruction occupies an SM sub-partition for 64 clocks whatever its active lanes, so the time
 // of a step is the number of FP64 instructions of a warp. G = 8 lanes hold one particle as long as the
-// warps, four particles each, have sub-partitions of their own (kTabGroupBelow = 4 x 608): lanes 0
+// warps, four particles each, have sub-partitions of their own (up to 4 sub_partitions()): lanes 0
 // and 1 evaluate force and electron density and the nuclear density of one plane each at once, lanes 0 to 3 one RK4 stage's longitudinal
 // velocity each, every lane draws the kicks of one of the next eight steps, and the lanes share the
 // record's stores. G = 1 beyond.
 // ------------------------------------------------------------------------------------
 constexpr int kTabI = 256, kTabDeg = 11, kTabC = kTabDeg + 1;
 constexpr int kTabThreads = 128;
-constexpr int64_t kTabGroupBelow = 2432;
 constexpr size_t kTabBytes = sizeof(double) * 2 * kTabI * kTabC;
 
 // The polynomials resolve the fit. A Gaussian of e^{-k r^2} leaves out, at half an interval of h = d_p / kTabI, at most
@@ -1583,8 +1591,6 @@ __device__ __forceinline__ float planar_force32(const Chan32 &C, const Planar32 
 // j < 2K evaluates plane j's sum over the terms and the planes are added in order from the lanes' values, so
 // the force is the one-lane form's, bit for bit.
 constexpr int kGroup32 = 8;
-// a warp, four particles, per SM sub-partition
-constexpr int64_t kGroup32Below = 4 * 608 + 1;
 
 __device__ __forceinline__ float planar_force32_group(const Chan32 &C, const Planar32 &P, float sw, int gl, unsigned mask) {
   int jlo;
@@ -1912,7 +1918,8 @@ int launch_trajectories(const rad_channel *ch, const rad_planar_potential *pot, 
   C.ms_loss = (ch->flags & RAD_TRAJ_MS_LOSS) != 0;
   // one thread per particle; small ensembles spread one warp per SM (the integration is a
   // dependent chain per thread), large ones fill the SMs with 128-thread blocks
-  const int block = n_particles < 152 * 4 * 32 ? 32 : 128;
+  const int64_t subs = sub_partitions();
+  const int block = n_particles < subs * 32 ? 32 : 128;
   int64_t grid = (n_particles + block - 1) / block;
   if (grid > 1 << 20) grid = 1 << 20;
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -1942,7 +1949,7 @@ int launch_trajectories(const rad_channel *ch, const rad_planar_potential *pot, 
     M.ms = C.ms;
     M.ll = C.ll;
     M.ms_loss = C.ms_loss;
-    if (pot && P32.K <= kGroup32 / 2 && n_particles < kGroup32Below)
+    if (pot && P32.K <= kGroup32 / 2 && n_particles <= 4 * subs)
       k_channel_mixed<true, kGroup32><<<static_cast<unsigned>((n_particles * kGroup32 + 31) / 32), 32, 0, st>>>(
           M, P32, n_particles, offsets, n_samples_total, energy_eV, x0, thx0, thy0, particle_ids, seed, out,
           energy_out, ds);
@@ -1955,14 +1962,15 @@ int launch_trajectories(const rad_channel *ch, const rad_planar_potential *pot, 
           M, P32, n_particles, offsets, n_samples_total, energy_eV, x0, thx0, thy0, particle_ids, seed, out,
           energy_out, ds);
   } else if (pot && tab_fits(P, C)) {
-    const bool eight = n_particles < kTabGroupBelow;
+    const bool eight = n_particles <= 4 * subs;
     auto kern = eight ? k_channel_tab<8> : k_channel_tab<1>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kTabBytes));
     if (e != cudaSuccess) return cuda_status(e);
     // one block per SM as long as its 128 threads hold the particles, else up to three
     const int64_t per_block = eight ? kTabThreads / 8 : kTabThreads;
     const int64_t blocks = (n_particles + per_block - 1) / per_block;
-    const int64_t tgrid = n_particles < 152 ? n_particles : blocks <= 152 ? 152 : blocks < 456 ? blocks : 456;
+    const int64_t sms = subs / 4;
+    const int64_t tgrid = n_particles < sms ? n_particles : std::min(std::max(blocks, sms), 3 * sms);
     kern<<<static_cast<unsigned>(tgrid), kTabThreads, kTabBytes, st>>>(C, P, n_particles, offsets, n_samples_total,
                                                                       energy_eV, x0, thx0, thy0, particle_ids, dt,
                                                                       seed, out, energy_out, ds);
@@ -2073,7 +2081,7 @@ int launch_axial(const rad_channel *ch, const rad_axial_potential *pot, int64_t 
   C.ms_loss = (ch->flags & RAD_TRAJ_MS_LOSS) != 0;
   if (n_particles < kGroupBelow) {  // lane groups share each particle's force evaluation
     const int block = 32;  // one-warp blocks, spread evenly over the SMs
-    const bool warp = n_particles < kWarpBelow;
+    const bool warp = n_particles <= sub_partitions();
     const int64_t grid = (n_particles * (warp ? 32 : kGroup) + block - 1) / block;
     auto kern = warp ? k_axial_group<32> : k_axial_group<16>;
     kern<<<static_cast<unsigned>(grid), block, 0, static_cast<cudaStream_t>(stream)>>>(
@@ -2142,7 +2150,8 @@ int launch_adaptive(const rad_channel *ch, const rad_planar_potential *pot, cons
   C.ll = (ch->flags & RAD_TRAJ_LL) != 0;
   C.ms_loss = (ch->flags & RAD_TRAJ_MS_LOSS) != 0;
   StepCtl S{sc->rtol, sc->atol_x, sc->atol_v, sc->max_level, sc->max_substeps};
-  const int block = n_particles < 152 * 4 * 32 ? 32 : 128;
+  const int64_t subs = sub_partitions();
+  const int block = n_particles < subs * 32 ? 32 : 128;
   int64_t grid = (n_particles + block - 1) / block;
   if (grid > 1 << 20) grid = 1 << 20;
   const cudaStream_t st = static_cast<cudaStream_t>(stream);

@@ -27,7 +27,7 @@ def check(got, off, picks, x0, th, E, L, dt, seed, charge, flags, orc, rho):
         assert np.all(err <= 1e-9), (p, err)
 
 
-@pytest.mark.parametrize("n,L", [(24, 300), (2432, 24), (4096, 12)])
+@pytest.mark.parametrize("n,L", [(24, 300), (2433, 24), (4096, 12)])
 @pytest.mark.parametrize("h2k", [0.0195, 0.0199, 0.05])
 @pytest.mark.parametrize("charge", [+1, -1])
 def test_narrow_terms(n, L, h2k, charge):

@@ -14,7 +14,7 @@ from test_crystal_gpu import D_P, MS, channel, potentials, run_gpu
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n", [24, 2432])
+@pytest.mark.parametrize("n", [24, 2433])
 def test_planar_kicks_between_the_planes(n):
     """Positrons entering parallel to the planes at 2 to 12.8 thermal amplitudes from the nearest one; eight lanes
     and one lane per particle."""
