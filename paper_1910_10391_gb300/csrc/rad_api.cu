@@ -239,13 +239,16 @@ int configure(rad_plan p, const Choice &c, bool moments = true) {
       p->cheb_scratch = nullptr;
       p->cheb_cap = 0;
       cudaError_t e = cudaMalloc(&p->cheb_scratch, bytes);
-      if (e != cudaSuccess) {  // no room: the direct kernel alone
+      if (e != cudaSuccess) {  // no room: the direct kernel alone, with its own split
         (void)cudaGetLastError();
-        p->nodes = false;
-      } else {
-        p->cheb_cap = bytes;
+        return configure(p, c, false);
       }
+      p->cheb_cap = bytes;
     }
+  } else if (p->cheb_scratch) {  // the partials may need its room
+    cudaFree(p->cheb_scratch);
+    p->cheb_scratch = nullptr;
+    p->cheb_cap = 0;
   }
   const size_t need = static_cast<size_t>(std::max<int64_t>(per_chunk * p->n_chunks, 1));
   if (need > p->part_cap) {

@@ -1,0 +1,62 @@
+"""Host side of plans without a device (fake_cudart.cpp): what they allocate, what they fall back to when memory is short."""
+import pytest
+
+import fake_gpu
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    return fake_gpu.library(str(tmp_path_factory.mktemp("fake")))
+
+
+# samples, particles, energies, directions, model, precision (0 FP64, 2 double-float)
+SHAPES = [(40961, 1, 512, 225, 0, 0), (40961, 1, 512, 225, 0, 2), (32000, 64, 192, 324, 2, 0), (72000, 6, 384, 576, 2, 2)]
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_short_memory_falls_back_to_the_direct_kernel(fake, shape):
+    """The moment kernel's scratch or its finer split do not fit: the plan is the direct kernel's, with its split and nothing
+    held for the moment kernel, wherever that plan fits."""
+    out = fake_gpu.run(fake, f"""
+shape = {shape}
+def sizes(cut):
+    rc, h = f.plan(*shape)
+    assert rc == 0
+    assert f.lib.rad_plan_set_cut(h, cut) == 0
+    d = f.describe(h)
+    f.launches(h)  # the library's own tables are there from now on
+    f.lib.rad_plan_destroy(h)
+    return d
+route, direct = sizes(shape[2]), sizes(0)
+assert route["cut"] != "0" and direct["cut"] == "0"
+# what a plan of the direct kernel alone needs, from the least capacity that admits one
+lo, hi = 0, 1 << 36
+while hi - lo > 1:
+    mid = (lo + hi) // 2
+    f.lib.fake_capacity(mid)
+    rc, h = f.plan(*shape)
+    f.lib.rad_plan_destroy(h) if rc == 0 else None
+    lo, hi = (lo, mid) if rc == 0 else (mid, hi)
+least = hi
+ncomp = 8 if shape[4] == 2 else 6
+parts = int(direct["chunks"]) * shape[2] * shape[3] * (ncomp if direct["amp"] == "1" else 1) * 8
+need = f.lib.fake_used() + parts + shape[2] * shape[3] * 8 + 4096
+assert least <= need, (least, need)
+seen = set()
+for k in range(64):  # capacities up to beyond the moment kernel's needs
+    f.lib.fake_capacity(least + k * (1 << 24))
+    rc, h = f.plan(*shape)
+    assert rc == 0
+    d = f.describe(h)
+    assert f.lib.fake_used() <= least + k * (1 << 24)
+    if d["cut"] == "0":
+        assert {{q: d[q] for q in ("chunks", "amp", "nq", "R")}} == {{q: direct[q] for q in ("chunks", "amp", "nq", "R")}}, (k, d, direct)
+        assert f.lib.fake_used() <= need
+    seen.add(d["cut"])
+    n, m = f.launches(h)
+    assert n == m, (n, m)
+    f.lib.rad_plan_destroy(h)
+    assert f.lib.fake_used() <= 1 << 20
+print(sorted(seen), least, need)
+""")
+    print(out)
