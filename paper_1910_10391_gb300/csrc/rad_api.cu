@@ -118,6 +118,45 @@ constexpr int64_t kChebMinFp64 = 24, kChebMinDf = 64;
 // Partials that a finer split for the moment kernel may take (doubles).
 constexpr int64_t kChebPartials = int64_t(1) << 26;
 
+// Costs of the plan's node or moment kernel, for the choice of the cut.
+NodeCost route_cost(rad_plan p) {
+  NodeCost nc;
+  if (p->precision == RAD_MIXED) {
+    nc = node_cost(p->mode, p->n_omega, p->shape.R);
+    const int64_t items = node_tiles(p->n_omega) * p->n_angles * p->n_chunks, slots = 4LL * p->sms;
+    if (items > 0 && items < slots) nc.scale(static_cast<float>(slots) / static_cast<float>(items));
+  } else {
+    const bool df = p->precision == RAD_FP64_DF;
+    nc = cheb_cost(p->mode, df, 32 * p->shape.R * (df ? p->shape.NW : 1));
+    // idle lanes of the last direction tile cost as much as the others
+    const float waste = static_cast<float>((p->n_angles + 31) / 32 * 32) / static_cast<float>(p->n_angles);
+    const int64_t items = cheb_tiles(p->mode, p->n_omega, p->n_angles) * p->n_chunks;
+    if (p->n_particles > 0)
+      nc.cap = static_cast<float>(std::max<int64_t>(std::min<int64_t>(256, p->n_samples_total / p->n_particles / p->n_q), 1));
+    const int64_t slots = df ? 2LL * p->sms : p->sms;
+    nc.scale(waste * (items < slots ? static_cast<float>(slots) / static_cast<float>(items) : 1.f));
+  }
+  nc.set_cut = p->set_cut;
+  return nc;
+}
+
+// Whether any number of energies could be worth the node or moment kernel, whatever the trajectories: with runs of the
+// largest length, whole tiles at a time and the last one up to the end. What this excludes, the choice on the device
+// (node_plan in rad_post.cu, with the same costs and margin) leaves to the direct kernel in every call.
+bool route_may_pay(const NodeCost &nc, int64_t n_omega) {
+  const double direct = 1.001 * kRouteMargin * nc.direct * static_cast<double>(n_omega);
+  double total = 0.0;
+  for (int64_t e0 = 0; e0 < n_omega && total < direct; e0 += nc.tile) {
+    const int64_t n = std::min<int64_t>(nc.tile, n_omega - e0), g = std::min<int64_t>(nc.gran, n);
+    auto part = [&](int64_t k) { return nc.fixed + (nc.per_run + nc.per_energy * static_cast<double>(k)) / nc.cap; };
+    // linear in the number of energies taken from this tile: its ends decide
+    for (int64_t k : {g, n})
+      if (total + part(k) + nc.direct * static_cast<double>(n_omega - e0 - k) < direct) return true;
+    total += part(n);
+  }
+  return false;
+}
+
 // Work decomposition for a choice; (re)allocates scratch when it grows.
 // `moments` false: without the node or moment kernel.
 int configure(rad_plan p, const Choice &c, bool moments = true) {
@@ -231,6 +270,10 @@ int configure(rad_plan p, const Choice &c, bool moments = true) {
   p->choice = c;
   p->nodes = p->precision == RAD_MIXED ? moments && c.pp && def_shape && node_path_allowed(sh, p->n_omega, p->n_angles, p->n_chunks)
                                        : cheb && ctiles <= (INT32_MAX - 65536) / p->n_chunks;
+  if (p->nodes && p->set_cut < 0 && !route_may_pay(route_cost(p), p->n_omega)) {
+    if (p->precision != RAD_MIXED) return configure(p, c, false);
+    p->nodes = false;
+  }
   if (p->precision != RAD_MIXED && p->nodes) {
     p->cheb_grid = static_cast<int>(std::min<int64_t>(ctiles * p->n_chunks, cheb_res));
     const size_t bytes = cheb_scratch_bytes(p->mode, p->n_omega, p->cheb_grid);
@@ -378,23 +421,7 @@ int execute(rad_plan p, const double *samples, const int64_t *offsets, const dou
   Params P = make_params(p, samples, offsets, gamma, energy, weight, hw, tx, ty, table);
   e = cudaMemsetAsync(p->ctrl, 0, kCtrlBytes, st);
   if (e != cudaSuccess) return cuda_fail(e);
-  NodeCost nc;
-  if (p->nodes && p->precision == RAD_MIXED) {
-    nc = node_cost(p->mode, p->n_omega, p->shape.R);
-    const int64_t items = node_tiles(p->n_omega) * p->n_angles * p->n_chunks, slots = 4LL * p->sms;
-    if (items < slots) nc.scale(static_cast<float>(slots) / static_cast<float>(items));
-  } else if (p->nodes) {
-    const bool df = p->precision == RAD_FP64_DF;
-    nc = cheb_cost(p->mode, df, 32 * p->shape.R * (df ? p->shape.NW : 1));
-    // idle lanes of the last direction tile cost as much as the others
-    const float waste = static_cast<float>((p->n_angles + 31) / 32 * 32) / static_cast<float>(p->n_angles);
-    const int64_t items = cheb_tiles(p->mode, p->n_omega, p->n_angles) * p->n_chunks;
-    if (p->n_particles > 0)
-      nc.cap = static_cast<float>(std::max<int64_t>(std::min<int64_t>(256, p->n_samples_total / p->n_particles / p->n_q), 1));
-    const int64_t slots = df ? 2LL * p->sms : p->sms;
-    nc.scale(waste * (items < slots ? static_cast<float>(slots) / static_cast<float>(items) : 1.f));
-  }
-  nc.set_cut = p->set_cut;
+  const NodeCost nc = p->nodes ? route_cost(p) : NodeCost{};
   p->ran = true;
   e = launch_validate(P, d_omega, need_dom, bin_of_angle, nc, st);
   if (e != cudaSuccess) return cuda_fail(e);

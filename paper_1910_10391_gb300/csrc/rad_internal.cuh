@@ -273,6 +273,8 @@ struct NodeCost {
     per_energy *= f;
   }
 };
+// The route has to promise a fifth less than the direct sum (see node_plan in rad_post.cu).
+constexpr float kRouteMargin = 0.8f;
 NodeCost node_cost(int mode, int64_t n_omega, int direct_r);
 int64_t node_tiles(int64_t n_omega);  // energy tiles of the node kernel
 cudaError_t launch_mixed_nodes(const Params &P, const float *prep, int sms, cudaStream_t st);

@@ -75,7 +75,7 @@ __device__ void node_plan(const Params &P, const NodeCost &c_) {
   };
   // the route has to promise a fifth less than the direct sum: the estimate is that good (over 110 drawn
   // calls of the library's ranges the slowest came out 7 % slower than directly, a call of half a ms)
-  float best = 0.8f * c_.direct * static_cast<float>(P.n_omega), done = 0.f;  // done: whole tiles below
+  float best = kRouteMargin * c_.direct * static_cast<float>(P.n_omega), done = 0.f;  // done: whole tiles below
   // at most some hundred steps: beyond 64 tiles whole groups of them are taken at once
   const int64_t group = (P.n_omega + 64 * static_cast<int64_t>(c_.tile) - 1) / (64 * static_cast<int64_t>(c_.tile));
   const int64_t tile = c_.tile * group, gran = group > 1 ? tile : c_.gran;

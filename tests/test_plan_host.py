@@ -60,3 +60,37 @@ for k in range(64):  # capacities up to beyond the moment kernel's needs
 print(sorted(seen), least, need)
 """)
     print(out)
+
+
+# samples, particles, energies, directions, model, precision: few work items, so that the moment or node kernel would leave
+# most of the SMs idle, or too few energies for its fixed cost
+SMALL = [(1478, 7, 80, 16, 2, 0), (1478, 7, 80, 33, 2, 2), (340, 2, 512, 16, 0, 0), (340, 2, 513, 16, 0, 2), (1031, 1, 130, 40, 2, 2),
+         (1468, 4, 129, 25, 0, 1), (2999, 1, 160, 16, 2, 1), (512, 1, 96, 16, 0, 1), (4000, 2, 24, 16, 0, 0)]
+LARGE = [(4096, 1, 128, 256, 0, 0), (4096, 1, 128, 256, 0, 1), (40961, 1, 500, 225, 0, 2), (32000, 64, 192, 324, 2, 0),
+         (72000, 6, 384, 576, 2, 2), (640000, 32, 512, 4096, 0, 1), (524288, 64, 256, 512, 2, 1)]
+
+
+def test_calls_that_cannot_gain_are_the_direct_kernels(fake):
+    """Where the costs exclude the route whatever the trajectories, a plan has the direct kernel's split, memory and number
+    of launches; the calls of the library's workloads keep the route."""
+    fake_gpu.run(fake, f"""
+for shape in {SMALL}:
+    found = []
+    for cut in (-1, 0):
+        rc, h = f.plan(*shape)
+        assert rc == 0
+        assert f.lib.rad_plan_set_cut(h, cut) == 0
+        d, n = f.describe(h), f.launches(h)
+        assert n[0] == n[1]
+        used = f.lib.fake_used()
+        f.lib.rad_plan_destroy(h)
+        found.append((d, n, used - f.lib.fake_used()))
+    assert found[0] == found[1], (shape, found)
+    assert found[0][0]["cut"] == "0"
+for shape in {LARGE}:
+    rc, h = f.plan(*shape)
+    assert f.describe(h)["cut"] == "auto", shape
+    n = f.launches(h)
+    assert n[0] == n[1]
+    f.lib.rad_plan_destroy(h)
+""")
