@@ -276,8 +276,8 @@ int rad_plan_set_sincos_split(rad_plan plan, int every);
  * rad_plan_set_cut -- how many of the lowest photon energies are summed over runs of samples
  * (RAD_MIXED: equispaced frequency nodes; RAD_FP64, RAD_FP64_DF: Chebyshev moments) instead of
  * term by term. n_lowest = -1 (a new plan's setting): chosen on the device in every call, from
- * the kernels' costs. 0: none. Otherwise n_omega or a multiple of the energies of one work
- * item of the term-by-term kernel (32 R; RAD_FP64_DF 32 R NW). It applies while the
+ * the kernels' costs. 0: none. Otherwise n_omega or a multiple of the energies that the
+ * term-by-term kernel takes together (32 R; RAD_FP64_DF 128). It applies while the
  * plan has the launch shape that a new plan of its size has; energies that do not ascend are
  * summed term by term whatever is set. RAD_EINVAL for other values, and for n_lowest > 0
  * where the plan has no such kernel: RAD_MIXED below 96 energies or without its pre-pass,

@@ -48,10 +48,12 @@ struct rad_plan_s {
   int32_t n_bins = 0;
   Choice choice{};
   LaunchShape shape{};
+  LaunchShape other{};  // RAD_FP64_DF with the moment kernel: k_df's other energies per lane, which the cut may leave a better number for
   int n_wt = 0, n_nt = 0, amp_mode = 0, n_q = 1;
   bool nodes = false;  // the lowest energies may go through the frequency-node or moment kernel
   int64_t set_cut = -1;  // how many of them: as asked for (rad_plan_set_cut), or by the costs (-1)
   bool ran = false;
+  bool df_filled = true;
   int cheb_grid = 0;   // resident blocks of the moment kernel (FP64 forms)
   unsigned char *cheb_scratch = nullptr;
   size_t cheb_cap = 0;
@@ -90,15 +92,20 @@ ShapeKey key_of(int dev, int64_t ns, int64_t np, int64_t no, int64_t na, int mod
 // Defaults before any autotuning: the fastest shapes on the 10 GeV positron ensemble (512 hw x
 // 64 x 64 directions, 32 particles per launch). The mixed kernel runs 8 warps per block, 2 blocks
 // per SM; spin-1/2 keeps every sin/cos on the SFU, classical and spin-0 (two fewer sums per term)
-// take 1/8 of them on the FMA pipe. k_df's blocks of 4 warps take 128 energies of one
-// direction: the moment kernel takes the lowest ones in steps of as many, and 256 per block (3 to 5 %
-// faster per term, and taken where one such block holds all energies) left half of a block idle for the
-// 128 highest of 384.
-Choice default_choice(int precision, int mode, int64_t n_omega) {
+// take 1/8 of them on the FMA pipe. k_df's blocks of 4 warps take 128 or 256 energies of one direction (df_energies).
+Choice default_choice(int precision, int mode, int64_t n_omega, bool df_filled) {
   if (precision == RAD_FP64) return Choice{2, 8, 64, 1, 0};
-  if (precision == RAD_FP64_DF) return Choice{n_omega > 128 && n_omega <= 256 ? 2 : 1, 4, 64, 1, 0};
+  if (precision == RAD_FP64_DF) return Choice{df_energies(n_omega, df_filled), 4, 64, 1, 0};
   if (mode == RAD_SPIN_HALF) return Choice{2, 8, 256, 1, 1, 0};
   return Choice{2, 8, 256, 1, 1, 6};
+}
+
+// k_df's blocks of 256 energies fill the GPU: 64 of them and, with the pieces that the trajectories can be cut into, 900 (over
+// 115 calls of 4 to 400 directions, 1 to 64 particles of 500 to 20000 samples, 256 energies per block were 0.99 to 1.15
+// times as fast from there on and 0.6 to 1.08 below)
+bool df_fills(int64_t ns, int64_t np, int64_t no, int64_t na) {
+  const int64_t tiles = (no + 255) / 256 * na, pieces = np > 0 ? np * std::max<int64_t>(ns / np / 128, 1) : 1;
+  return tiles >= 64 && (tiles >= 900 || tiles * pieces >= 900);
 }
 
 bool supported(int precision, const Choice &c) {
@@ -127,7 +134,7 @@ NodeCost route_cost(rad_plan p) {
     if (items > 0 && items < slots) nc.scale(static_cast<float>(slots) / static_cast<float>(items));
   } else {
     const bool df = p->precision == RAD_FP64_DF;
-    nc = cheb_cost(p->mode, df, 32 * p->shape.R * (df ? p->shape.NW : 1));
+    nc = cheb_cost(p->mode, df, df ? 128 : 32 * p->shape.R);
     // idle lanes of the last direction tile cost as much as the others
     const float waste = static_cast<float>((p->n_angles + 31) / 32 * 32) / static_cast<float>(p->n_angles);
     const int64_t items = cheb_tiles(p->mode, p->n_omega, p->n_angles) * p->n_chunks;
@@ -185,7 +192,7 @@ int configure(rad_plan p, const Choice &c, bool moments = true) {
   const bool per_particle = (p->want & RAD_PER_PARTICLE) != 0;
   // the node and moment forms go with the default launch shape; a caller that sets another asks for
   // that direct kernel
-  const Choice def = default_choice(p->precision, p->mode, p->n_omega);
+  const Choice def = default_choice(p->precision, p->mode, p->n_omega, p->df_filled);
   const bool def_shape = c.R == def.R && c.NW == def.NW && c.T == def.T && c.pp == def.pp;
   const bool df = p->precision == RAD_FP64_DF;
   moments &= p->set_cut != 0;
@@ -275,6 +282,13 @@ int configure(rad_plan p, const Choice &c, bool moments = true) {
     p->nodes = false;
   }
   if (p->precision != RAD_MIXED && p->nodes) {
+    if (df) {  // the energies above the cut may suit the other number per lane: both are launched, one works
+      p->other = LaunchShape{3 - c.R, c.NW, c.T, 0, 0, 0};
+      const int64_t res = static_cast<int64_t>(p->sms) * occupancy_df(p->other, p->mode), per = 32LL * p->other.R * c.NW;
+      const int64_t items = (p->n_omega + per - 1) / per * p->n_angles * p->n_chunks;
+      if (res <= 0 || items > static_cast<int64_t>(INT32_MAX) - res) return configure(p, c, false);
+      p->other.grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(items, res)));
+    }
     p->cheb_grid = static_cast<int>(std::min<int64_t>(ctiles * p->n_chunks, cheb_res));
     const size_t bytes = cheb_scratch_bytes(p->mode, p->n_omega, p->cheb_grid);
     if (bytes > p->cheb_cap) {
@@ -373,6 +387,7 @@ Params make_params(rad_plan p, const double *samples, const int64_t *offsets, co
                    : nullptr;
   P.node_cut = p->nodes ? p->ctrl + 2 : nullptr;
   P.counter2 = p->ctrl + 3;
+  P.df_filled = p->df_filled;
   return P;
 }
 
@@ -443,6 +458,10 @@ int execute(rad_plan p, const double *samples, const int64_t *offsets, const dou
     e = launch_fp64(P, &sh, st);
   } else if (p->precision == RAD_FP64_DF) {
     e = launch_df(P, &sh, st);
+    if (e == cudaSuccess && p->nodes) {
+      sh = p->other;
+      e = launch_df(P, &sh, st);
+    }
   } else if (p->choice.pp) {
     if (p->nodes) {
       e = launch_mixed_nodes(P, p->prep, p->sms, st);
@@ -506,7 +525,8 @@ int plan_create(int64_t ns, int64_t np, int64_t no, int64_t na, int mode, int pr
     delete p;
     return cuda_fail(e);
   }
-  Choice c = default_choice(prec, mode, no);
+  p->df_filled = df_fills(ns, np, no, na);
+  Choice c = default_choice(prec, mode, no, p->df_filled);
   {
     std::lock_guard<std::mutex> lk(g_mu);
     auto it = g_tuned.find(key_of(dev, ns, np, no, na, mode, prec, want, p->n_bins));
@@ -636,7 +656,7 @@ int rad_plan_set_sincos_split(rad_plan plan, int every) {
 
 int rad_plan_set_cut(rad_plan plan, int64_t n_lowest) {
   if (!plan || n_lowest < -1 || n_lowest > plan->n_omega) return RAD_EINVAL;
-  const int64_t gran = 32LL * plan->choice.R * (plan->precision == RAD_FP64_DF ? plan->choice.NW : 1);
+  const int64_t gran = plan->precision == RAD_FP64_DF ? 128 : 32LL * plan->choice.R;
   if (n_lowest > 0 && n_lowest < plan->n_omega && n_lowest % gran != 0) return RAD_EINVAL;
   const int64_t old = plan->set_cut;
   plan->set_cut = n_lowest;
@@ -700,8 +720,9 @@ int rad_plan_last_kernel_ms(rad_plan plan, double *ms) {
 int rad_plan_kernel_launches(rad_plan plan) {
   if (!plan) return 0;
   if (plan->n_omega == 0 || plan->n_angles == 0) return 0;
-  // pre-pass; node or moment kernel
-  const int pre = (plan->precision == RAD_MIXED && plan->choice.pp ? 1 : 0) + (plan->nodes ? 1 : 0);
+  // pre-pass; node or moment kernel, and k_df's other shape with it
+  const int pre = (plan->precision == RAD_MIXED && plan->choice.pp ? 1 : 0) +
+                  (plan->nodes ? (plan->precision == RAD_FP64_DF ? 2 : 1) : 0);
   if (plan->want & RAD_PER_PARTICLE) return 3 + pre;  // validate, main, per-particle reduce
   int n = 3 + pre;  // validate, main, finalize
   if (plan->want & 6) n += 1;

@@ -89,15 +89,14 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 5 : 2) k_df(const Params P)
   int *s_item = reinterpret_cast<int *>(sm + L::kMisc);
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // energies below node_cut (a multiple of NW 32 R, or all of them) are summed by k_cheb; the first tile above
-  // it stays in shared memory, out of the term loop's registers
+  // energies below node_cut are summed by k_cheb; it stays in shared memory, out of the term loop's registers
   if (tid == 0) {
-    const int64_t cut = P.node_cut ? *P.node_cut : 0;
     s_item[1] = *reinterpret_cast<volatile int *>(P.status);
-    s_item[2] = static_cast<int>((cut + NW * 32 * R - 1) / (NW * 32 * R));
+    s_item[2] = P.node_cut ? *P.node_cut : 0;
   }
   __syncthreads();
-  if (s_item[1] != 0) return;
+  if (s_item[1] != 0 || s_item[2] >= P.n_omega) return;
+  if (P.node_cut && df_energies(P.n_omega - s_item[2], P.df_filled) != R) return;  // the other launch's
 
   // (cos, sin)(2 pi j / 2048) as float pairs (c_hi, c_lo, s_hi, s_lo) from every other entry of the
   // FP64 table (2048 entries, 32 KB)
@@ -115,7 +114,6 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 5 : 2) k_df(const Params P)
   float4 *sFa = reinterpret_cast<float4 *>(sm + L::kNk + T * 8);   // (fx_hi, fx_lo, fy_hi, fy_lo)
   float2 *sFj = reinterpret_cast<float2 *>(sm + L::kNk + T * 24);  // (j_hi, j_lo), spin 1/2 only
 
-  if (s_item[2] >= P.n_wt) return;
   int s = 0;
 
   for (;;) {
@@ -123,21 +121,21 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? 5 : 2) k_df(const Params P)
     __syncthreads();
     const int64_t item = s_item[0];
     __syncthreads();
-    const int wt0 = s_item[2], n_wt = P.n_wt - wt0;
-    const int64_t per_chunk = static_cast<int64_t>(n_wt) * P.n_nt;
+    const int64_t n_wt = (P.n_omega - s_item[2] + NW * 32 * R - 1) / (NW * 32 * R);
+    const int64_t per_chunk = n_wt * P.n_nt;
     if (item >= per_chunk * P.n_chunks) break;
     const int64_t chunk = item / per_chunk;
     const int64_t rem = item % per_chunk;
     // one direction per item, shared by the block's warps (the per-sample preparation is done
-    // once for all of them); warp w takes the energies (wt NW + w) 32 R + 32 r + lane
+    // once for all of them); warp w takes the energies cut + (wt NW + w) 32 R + 32 r + lane
     const int64_t jdir = rem / n_wt;
-    const int wt = wt0 + static_cast<int>(rem % n_wt);
+    const int64_t wt = rem % n_wt;
     const double nx = P.theta_x[jdir];
     const double ny = P.theta_y[jdir];
     const double th2h = __dmul_rn(__dadd_rn(__dmul_rn(nx, nx), __dmul_rn(ny, ny)), 0.5);
 
     // energy indices; the energies themselves are read where they are used
-    const int64_t iw0 = (static_cast<int64_t>(wt) * NW + warp) * 32 * R + lane;
+    const int64_t iw0 = s_item[2] + (wt * NW + warp) * 32 * R + lane;
     auto hw_of = [&](int r) { return iw0 + 32 * r < P.n_omega ? __ldg(P.hw + iw0 + 32 * r) : 1.0; };
     double S_acc[R];
     double amp[R][NA];

@@ -74,6 +74,7 @@ struct Params {
   // launch)
   int *node_cut;
   int *counter2;
+  bool df_filled;  // RAD_FP64_DF: see df_energies
   double phase_budget;  // RAD_MIXED: largest accepted in-tile phase-offset bound (radians)
 };
 
@@ -280,6 +281,14 @@ int64_t node_tiles(int64_t n_omega);  // energy tiles of the node kernel
 cudaError_t launch_mixed_nodes(const Params &P, const float *prep, int sms, cudaStream_t st);
 
 // FP64-accurate kernel with double-float FP32 arithmetic after the FP64 phase (rad_df.cu)
+// Energies per lane of k_df's blocks of 4 warps for n energies. 2 (256 of one direction per block) are up to 10 % faster per
+// term where the blocks fill the GPU (`filled`: 512 energies x 576 directions 46.2 against 47.9 ms), unless they leave half of a
+// block idle: an odd number of 128s (384 energies 68 against 56 ms), up to 12 of them. Below that many blocks 128 per
+// block give twice as many (512 energies x 16 directions x 340 samples 88 against 147 us).
+__host__ __device__ inline int df_energies(int64_t n, bool filled) {
+  const int64_t blocks = (n + 127) / 128;
+  return blocks == 2 || (filled && (blocks % 2 == 0 || blocks > 12)) ? 2 : 1;
+}
 bool shape_supported_df(int R, int NW, int T);
 int occupancy_df(const LaunchShape &s, int mode = RAD_SPIN_HALF);
 cudaError_t launch_df(const Params &P, LaunchShape *shape, cudaStream_t st);

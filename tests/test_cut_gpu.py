@@ -165,3 +165,19 @@ def test_refused_settings():
     few = rad.DeviceInputs(tr, directions(15, I.omega_log(200, 1e5, 4e8)))
     q, _ = plan_of(few, rad.RAD_SPIN_HALF, rad.RAD_FP64)
     assert q.set_cut(few.n_omega) == rad.RAD_EINVAL
+
+
+@pytest.mark.parametrize("mode", [rad.RAD_CLASSICAL, rad.RAD_SPIN_HALF])
+@pytest.mark.parametrize("n_omega", [600, 640])
+def test_double_float_energies_above_the_cut(mode, n_omega):
+    """k_df starts at the cut and takes one or two energies per lane by how many 128s are left above it: every number of them
+    from five down."""
+    tr, grid = bunch([300, 41]), directions(17, I.omega_log(n_omega, 1e5, 5e8))
+    ref = O.spectrum_cube(tr, grid, MODE_ORC[mode])
+    inp = rad.DeviceInputs(tr, grid)
+    p, _ = plan_of(inp, mode, rad.RAD_FP64_DF)
+    for cut in range(0, n_omega, 128):
+        assert p.set_cut(cut) == rad.RAD_OK
+        assert_fp64_close(cube_of(p, inp), ref)
+        assert p.last_cut() == cut
+    p.close()

@@ -94,3 +94,19 @@ for shape in {LARGE}:
     assert n[0] == n[1]
     f.lib.rad_plan_destroy(h)
 """)
+
+
+def test_double_float_energies_per_lane(fake):
+    """Two energies per lane unless that leaves half of a block idle or the GPU unfilled: calls that stay with the direct
+    kernel lose nothing to the moment kernel's granularity of 128."""
+    fake_gpu.run(fake, """
+for n, R in ((1, 1), (64, 1), (128, 1), (129, 2), (256, 2), (257, 1), (300, 1), (384, 1), (385, 2), (512, 2), (1024, 2), (1536, 2),
+             (1537, 2), (1280 + 128, 1), (1664, 2)):
+    for angles, samples, want in ((64, 4000, R), (4, 4000, R if n <= 256 else 1), (40, 400, R if n <= 256 else 1)):
+        rc, h = f.plan(samples, 2, n, angles, 0, 2)
+        assert rc == 0
+        assert f.lib.rad_plan_set_cut(h, 0) == 0
+        assert f.describe(h)["R"] == str(want), (n, angles, samples, f.describe(h))
+        assert f.launches(h)[0] == f.launches(h)[1] == 3
+        f.lib.rad_plan_destroy(h)
+""")
