@@ -228,8 +228,8 @@ int rad_plan_execute(rad_plan plan, const double *samples, const int64_t *offset
 
 /*
  * rad_plan_autotune -- times the plan's candidate launch shapes (frequencies per
- * thread, warps per block, time-tile length, work split) on the given inputs for at
- * most about budget_ms milliseconds, keeps the fastest in the plan and in the
+ * thread, warps per block, time-tile length, work split) on the given inputs, its current one
+ * first, for at most about budget_ms milliseconds, keeps the fastest in the plan and in the
  * library's tuning cache (used by rad_spectrum for the same shape). Synchronous.
  * Writes to the outputs (they hold a valid result of the chosen shape on return).
  */

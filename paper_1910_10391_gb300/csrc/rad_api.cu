@@ -741,7 +741,9 @@ int rad_plan_autotune(rad_plan plan, const double *samples, const int64_t *offse
                       double *out_bins, int budget_ms, void *stream) {
   if (!plan || budget_ms < 0) return RAD_EINVAL;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  std::vector<Choice> cands;
+  // the plan's own choice first: only it may have the node or moment kernel, and a budget that ends early must not
+  // leave a slower shape
+  std::vector<Choice> cands{plan->choice};
   const int Rs[] = {1, 2, 4};
   const int NWs[] = {4, 8};
   const int Ts[] = {64, 128, 256};
@@ -754,7 +756,7 @@ int rad_plan_autotune(rad_plan plan, const double *samples, const int64_t *offse
           for (int T : Ts)
             for (int m : mults) {
               Choice c{R, NW, T, m, pp, pe};
-              if (supported(plan->precision, c)) cands.push_back(c);
+              if (supported(plan->precision, c) && !same_choice(c, plan->choice)) cands.push_back(c);
             }
   const Choice start = plan->choice;
   Choice best = start;

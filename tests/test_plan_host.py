@@ -110,3 +110,16 @@ for n, R in ((1, 1), (64, 1), (128, 1), (129, 2), (256, 2), (257, 1), (300, 1), 
         assert f.launches(h)[0] == f.launches(h)[1] == 3
         f.lib.rad_plan_destroy(h)
 """)
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2])
+def test_autotune_times_the_current_choice_first(fake, precision):
+    """A budget that ends with the first candidate keeps the plan as it is."""
+    fake_gpu.run(fake, f"""
+rc, h = f.plan(640000, 32, 512, 4096, 0, {precision})
+assert rc == 0
+before = f.describe(h)
+assert before["cut"] == "auto"
+assert f.lib.rad_plan_autotune(h, *f.args(), 0, None) == 0
+assert f.describe(h) == before, (before, f.describe(h))
+""")
