@@ -125,24 +125,33 @@ constexpr int64_t kChebMinFp64 = 24, kChebMinDf = 64;
 // Partials that a finer split for the moment kernel may take (doubles).
 constexpr int64_t kChebPartials = int64_t(1) << 26;
 
+constexpr double kSecondKernelClocks = 50e3;
+
 // Costs of the plan's node or moment kernel, for the choice of the cut.
 NodeCost route_cost(rad_plan p) {
   NodeCost nc;
+  int64_t items, slots;  // of one energy tile; blocks that fill the GPU
   if (p->precision == RAD_MIXED) {
     nc = node_cost(p->mode, p->n_omega, p->shape.R);
-    const int64_t items = node_tiles(p->n_omega) * p->n_angles * p->n_chunks, slots = 4LL * p->sms;
-    if (items > 0 && items < slots) nc.scale(static_cast<float>(slots) / static_cast<float>(items));
+    items = p->n_angles * p->n_chunks;
+    slots = 4LL * p->sms;
   } else {
     const bool df = p->precision == RAD_FP64_DF;
     nc = cheb_cost(p->mode, df, df ? 128 : 32 * p->shape.R);
-    // idle lanes of the last direction tile cost as much as the others
-    const float waste = static_cast<float>((p->n_angles + 31) / 32 * 32) / static_cast<float>(p->n_angles);
-    const int64_t items = cheb_tiles(p->mode, p->n_omega, p->n_angles) * p->n_chunks;
-    if (p->n_particles > 0)
-      nc.cap = static_cast<float>(std::max<int64_t>(std::min<int64_t>(256, p->n_samples_total / p->n_particles / p->n_q), 1));
-    const int64_t slots = df ? 2LL * p->sms : p->sms;
-    nc.scale(waste * (items < slots ? static_cast<float>(slots) / static_cast<float>(items) : 1.f));
+    const int64_t lanes = (p->n_angles + 31) / 32 * 32;
+    nc.idle = static_cast<float>(lanes) / static_cast<float>(std::max<int64_t>(p->n_angles, 1));
+    items = lanes / 32 * p->n_chunks;
+    slots = df ? 2LL * p->sms : p->sms;
+    if (p->n_particles > 0) {
+      const int64_t piece = std::max<int64_t>(p->n_samples_total / p->n_particles / p->n_q, 1);
+      nc.setup /= static_cast<float>(piece);
+      nc.cap = static_cast<float>(std::min<int64_t>(256, piece));
+    }
   }
+  nc.slots = static_cast<float>(slots) / static_cast<float>(std::max<int64_t>(items, 1));
+  // a second kernel's start and end beside the first one's, in SM clocks per sample and direction
+  const double terms = static_cast<double>(std::max<int64_t>(p->n_samples_total, 1)) * static_cast<double>(std::max<int64_t>(p->n_angles, 1));
+  nc.second = static_cast<float>(kSecondKernelClocks * p->sms / terms);
   nc.set_cut = p->set_cut;
   return nc;
 }
@@ -155,11 +164,12 @@ bool route_may_pay(const NodeCost &nc, int64_t n_omega) {
   double total = 0.0;
   for (int64_t e0 = 0; e0 < n_omega && total < direct; e0 += nc.tile) {
     const int64_t n = std::min<int64_t>(nc.tile, n_omega - e0), g = std::min<int64_t>(nc.gran, n);
-    auto part = [&](int64_t k) { return nc.fixed + (nc.per_run + nc.per_energy * static_cast<double>(k)) / nc.cap; };
     // linear in the number of energies taken from this tile: its ends decide
     for (int64_t k : {g, n})
-      if (total + part(k) + nc.direct * static_cast<double>(n_omega - e0 - k) < direct) return true;
-    total += part(n);
+      if (nc.fill(static_cast<float>(e0 / nc.tile + 1)) * (total + nc.part(k, 1.f / nc.cap)) + nc.direct * static_cast<double>(n_omega - e0 - k) +
+              (e0 + k < n_omega ? nc.second : 0.f) < direct)
+        return true;
+    total += nc.part(n, 1.f / nc.cap);
   }
   return false;
 }

@@ -667,6 +667,7 @@ NodeCost cheb_cost(int mode, bool df, int direct_gran) {
   c.fixed = df ? (spin ? 36.f : 32.f) : 85.f;
   c.per_run = df ? 20.f : 110.f;
   c.per_energy = df ? (spin ? 17.f : 14.f) : (spin ? 58.f : 50.f);
+  c.setup = 11.f;  // once per piece, bessel_row: some 690 FP64 instructions per 32 energies, 16 clocks each, for 32 directions
   return c;
 }
 

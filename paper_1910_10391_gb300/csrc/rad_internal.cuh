@@ -267,11 +267,16 @@ struct NodeCost {
   int gran = 64, tile = 512, from_zero = 1, pow2 = 0;
   int64_t set_cut = -1;  // not chosen but asked for: so many energies, if they ascend
   float widen = 1.f, direct = 0.f, fixed = 0.f, per_run = 0.f, per_energy = 0.f, reach = 0.f, cap = 64.f;
-  // for a kernel that fills only a part of the SMs (or lanes) the costs rise by that factor
-  void scale(float f) {
-    fixed *= f;
-    per_run *= f;
-    per_energy *= f;
+  float setup = 0.f;   // per energy once in a piece (series coefficients), over the piece's samples
+  float second = 0.f;  // of a second kernel beside the route's
+  // `idle`: lanes of the last direction tile without a direction; `slots`: blocks that fill the GPU, per energy tile's items
+  float idle = 1.f, slots = 0.f;
+  // a route of so many energy tiles that fills only a part of the SMs (or lanes) costs that much more
+  __host__ __device__ float fill(float tiles) const { return idle * (slots > tiles ? slots / tiles : 1.f); }
+  // k energies of a tile at `runs` runs per sample
+  __host__ __device__ float part(int64_t k, float runs) const {
+    const float n = static_cast<float>(k);
+    return fixed + setup * n + (per_run + per_energy * n) * runs;
   }
 };
 // The route has to promise a fifth less than the direct sum (see node_plan in rad_post.cu).

@@ -80,7 +80,7 @@ __device__ void node_plan(const Params &P, const NodeCost &c_) {
   const int64_t group = (P.n_omega + 64 * static_cast<int64_t>(c_.tile) - 1) / (64 * static_cast<int64_t>(c_.tile));
   const int64_t tile = c_.tile * group, gran = group > 1 ? tile : c_.gran;
   int64_t cut = 0;
-  float lo = 0.f;
+  float lo = 0.f, tiles = static_cast<float>(group);  // tiles up to `end`
   for (int64_t e = 0; e < P.n_omega; e += gran) {
     const int64_t t0 = e / tile * tile;
     const int64_t end = e + gran < P.n_omega ? e + gran : P.n_omega;
@@ -89,14 +89,17 @@ __device__ void node_plan(const Params &P, const NodeCost &c_) {
     float runlen = fminf(fmaxf(c_.reach / fmaxf((ws(end - 1) - lo) * step, 1e-30f), 1.f), c_.cap);
     if (c_.pow2) runlen = exp2f(floorf(log2f(runlen)));
     const float runs = block_sum(cnt > 0.f ? 1.f / runlen : 0.f) / windows;
-    const float tiles = static_cast<float>(group);
-    const float part = tiles * c_.fixed + (tiles * c_.per_run + c_.per_energy * static_cast<float>(end - t0)) * runs;
-    const float total = done + part + c_.direct * static_cast<float>(P.n_omega - end);
+    const float part = c_.part(end - t0, runs) + static_cast<float>(group - 1) * (c_.fixed + c_.per_run * runs);
+    const float total = c_.fill(tiles) * (done + part) + c_.direct * static_cast<float>(P.n_omega - end) +
+                        (end < P.n_omega ? c_.second : 0.f);
     if (total < best) {
       best = total;
       cut = end;
     }
-    if (end == t0 + tile) done += part;
+    if (end == t0 + tile) {
+      done += part;
+      tiles += static_cast<float>(group);
+    }
   }
   if (tid == 0) *P.node_cut = static_cast<int>(cut);
 }
