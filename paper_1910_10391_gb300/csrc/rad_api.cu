@@ -125,7 +125,7 @@ constexpr int64_t kChebMinFp64 = 24, kChebMinDf = 64;
 // Partials that a finer split for the moment kernel may take (doubles).
 constexpr int64_t kChebPartials = int64_t(1) << 26;
 
-constexpr double kSecondKernelClocks = 50e3;
+constexpr double kSecondKernelClocks = 30e3;
 
 // Costs of the plan's node or moment kernel, for the choice of the cut.
 NodeCost route_cost(rad_plan p) {
@@ -135,13 +135,15 @@ NodeCost route_cost(rad_plan p) {
     nc = node_cost(p->mode, p->n_omega, p->shape.R);
     items = p->n_angles * p->n_chunks;
     slots = 4LL * p->sms;
+    nc.setup = p->mode == RAD_CLASSICAL ? 0.f : nc.setup * static_cast<float>(p->n_particles) /
+                                                    static_cast<float>(std::max<int64_t>(p->n_samples_total, 1));
   } else {
     const bool df = p->precision == RAD_FP64_DF;
     nc = cheb_cost(p->mode, df, df ? 128 : 32 * p->shape.R);
     const int64_t lanes = (p->n_angles + 31) / 32 * 32;
     nc.idle = static_cast<float>(lanes) / static_cast<float>(std::max<int64_t>(p->n_angles, 1));
     items = lanes / 32 * p->n_chunks;
-    slots = df ? 2LL * p->sms : p->sms;
+    slots = df ? 2LL * p->sms : 3LL * p->sms / 2;
     if (p->n_particles > 0) {
       const int64_t piece = std::max<int64_t>(p->n_samples_total / p->n_particles / p->n_q, 1);
       nc.setup /= static_cast<float>(piece);
@@ -160,13 +162,13 @@ NodeCost route_cost(rad_plan p) {
 // largest length, whole tiles at a time and the last one up to the end. What this excludes, the choice on the device
 // (node_plan in rad_post.cu, with the same costs and margin) leaves to the direct kernel in every call.
 bool route_may_pay(const NodeCost &nc, int64_t n_omega) {
-  const double direct = 1.001 * kRouteMargin * nc.direct * static_cast<double>(n_omega);
+  const double direct = 1.001 * nc.margin * nc.direct * static_cast<double>(n_omega);
   double total = 0.0;
   for (int64_t e0 = 0; e0 < n_omega && total < direct; e0 += nc.tile) {
-    const int64_t n = std::min<int64_t>(nc.tile, n_omega - e0), g = std::min<int64_t>(nc.gran, n);
+    const int64_t n = std::min<int64_t>(nc.tile, n_omega - e0), g = std::min<int64_t>(nc.gran, n), n0 = nc.tile;
     // linear in the number of energies taken from this tile: its ends decide
     for (int64_t k : {g, n})
-      if (nc.fill(static_cast<float>(e0 / nc.tile + 1)) * (total + nc.part(k, 1.f / nc.cap)) + nc.direct * static_cast<double>(n_omega - e0 - k) +
+      if (nc.spread(static_cast<float>(total) + nc.part(k, 1.f / nc.cap), nc.part(e0 > 0 ? n0 : k, 1.f / nc.cap)) + nc.direct * static_cast<double>(n_omega - e0 - k) +
               (e0 + k < n_omega ? nc.second : 0.f) < direct)
         return true;
     total += nc.part(n, 1.f / nc.cap);

@@ -660,7 +660,8 @@ NodeCost cheb_cost(int mode, bool df, int direct_gran) {
   c.gran = direct_gran;
   c.tile = cheb_tile(mode);
   c.cap = kWin;
-  c.widen = 1.6f;  // the widest of 32 directions, a row or more of a grid
+  c.tile_steps = 1;
+  c.widen = 1.05f;  // the widest of a window's steps against the widest of the 32 looked at
   c.reach = 0.95f * 2.f * static_cast<float>(spin ? (df ? Cheb<RAD_SPIN_HALF>::kPhi<true> : Cheb<RAD_SPIN_HALF>::kPhi<false>)
                                                      : (df ? Cheb<RAD_CLASSICAL>::kPhi<true> : Cheb<RAD_CLASSICAL>::kPhi<false>));
   c.direct = df ? (spin ? 1.45f : 1.3f) : (spin ? 11.5f : 9.6f);

@@ -265,22 +265,24 @@ bool node_path_allowed(const LaunchShape &s, int64_t n_omega, int64_t n_angles, 
 // `pow2`; `widen`: a block's widest direction against the mean.
 struct NodeCost {
   int gran = 64, tile = 512, from_zero = 1, pow2 = 0;
+  int tile_steps = 0;  // runs are bounded by the widest step over 32 directions, else by a direction's own
+  float margin = 0.9f;   // the share of the direct sum's cost that the route has to stay below
   int64_t set_cut = -1;  // not chosen but asked for: so many energies, if they ascend
   float widen = 1.f, direct = 0.f, fixed = 0.f, per_run = 0.f, per_energy = 0.f, reach = 0.f, cap = 64.f;
   float setup = 0.f;   // per energy once in a piece (series coefficients), over the piece's samples
+  int setup_if_differ = 0;  // only where the particles' energies differ
   float second = 0.f;  // of a second kernel beside the route's
-  // `idle`: lanes of the last direction tile without a direction; `slots`: blocks that fill the GPU, per energy tile's items
+  // `idle`: lanes of the last direction tile without a direction; `slots`: blocks that fill the GPU over one energy tile's
+  // work items, and over the share of the longest of them
   float idle = 1.f, slots = 0.f;
-  // a route of so many energy tiles that fills only a part of the SMs (or lanes) costs that much more
-  __host__ __device__ float fill(float tiles) const { return idle * (slots > tiles ? slots / tiles : 1.f); }
+  // tiles that cost `sum` together, the dearest `top`: below that many work items the GPU waits for the dearest ones
+  __host__ __device__ float spread(float sum, float top) const { return idle * (slots * top > sum ? slots * top : sum); }
   // k energies of a tile at `runs` runs per sample
   __host__ __device__ float part(int64_t k, float runs) const {
     const float n = static_cast<float>(k);
     return fixed + setup * n + (per_run + per_energy * n) * runs;
   }
 };
-// The route has to promise a fifth less than the direct sum (see node_plan in rad_post.cu).
-constexpr float kRouteMargin = 0.8f;
 NodeCost node_cost(int mode, int64_t n_omega, int direct_r);
 int64_t node_tiles(int64_t n_omega);  // energy tiles of the node kernel
 cudaError_t launch_mixed_nodes(const Params &P, const float *prep, int sms, cudaStream_t st);

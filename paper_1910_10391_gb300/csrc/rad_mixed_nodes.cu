@@ -594,6 +594,9 @@ NodeCost node_cost(int mode, int64_t n_omega, int direct_r) {
   c.direct = spin ? 1.0f / 7.6f : 1.0f / 8.5f;
   c.fixed = spin ? 8.5f : 6.8f;
   c.per_energy = spin ? 1.35f : 1.1f;
+  c.setup = 46.f;         // window values at a particle energy's w*: some 184 FP64 instructions a warp and 64 energies
+  c.margin = 0.85f;
+  c.setup_if_differ = 1;  // kept while the particle energy stays
   c.pow2 = 1;
   c.reach = static_cast<float>(56.0 * kPi);
   c.cap = 64.f;
