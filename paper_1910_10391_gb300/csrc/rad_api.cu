@@ -162,13 +162,14 @@ NodeCost route_cost(rad_plan p) {
 // largest length, whole tiles at a time and the last one up to the end. What this excludes, the choice on the device
 // (node_plan in rad_post.cu, with the same costs and margin) leaves to the direct kernel in every call.
 bool route_may_pay(const NodeCost &nc, int64_t n_omega) {
-  const double direct = 1.001 * nc.margin * nc.direct * static_cast<double>(n_omega);
+  auto items = [&](int64_t n) { return static_cast<double>((n + nc.gran - 1) / nc.gran * nc.gran); };
+  const double direct = 1.001 * nc.margin * nc.direct * items(n_omega);
   double total = 0.0;
   for (int64_t e0 = 0; e0 < n_omega && total < direct; e0 += nc.tile) {
     const int64_t n = std::min<int64_t>(nc.tile, n_omega - e0), g = std::min<int64_t>(nc.gran, n), n0 = nc.tile;
     // linear in the number of energies taken from this tile: its ends decide
     for (int64_t k : {g, n})
-      if (nc.spread(static_cast<float>(total) + nc.part(k, 1.f / nc.cap), nc.part(e0 > 0 ? n0 : k, 1.f / nc.cap)) + nc.direct * static_cast<double>(n_omega - e0 - k) +
+      if (nc.spread(static_cast<float>(total) + nc.part(k, 1.f / nc.cap), nc.part(e0 > 0 ? n0 : k, 1.f / nc.cap)) + nc.direct * items(n_omega - e0 - k) +
               (e0 + k < n_omega ? nc.second : 0.f) < direct)
         return true;
     total += nc.part(n, 1.f / nc.cap);

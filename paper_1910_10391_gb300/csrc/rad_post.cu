@@ -136,7 +136,9 @@ __device__ void node_plan(const Params &P, NodeCost c_) {
   // the route has to promise more than the estimate's error: over 46 calls of 1 to 25 particles, 20 to 676 directions and 63
   // to 1022 energies the chosen cut came out at most 5 % slower than the direct sum, 1.68 times as fast in the
   // geometric mean, and within 6 % of the best cut in all but one (16 %)
-  float best = c_.margin * c_.direct * static_cast<float>(P.n_omega), done = 0.f;  // done: whole tiles below
+  // energies of the direct kernel's work items, idle lanes of the last one among them
+  auto items = [&](int64_t n) { return static_cast<float>((n + c_.gran - 1) / c_.gran * c_.gran); };
+  float best = c_.margin * c_.direct * items(P.n_omega), done = 0.f;  // done: whole tiles below
   // at most some hundred steps: beyond 64 tiles whole groups of them are taken at once
   const int64_t group = (P.n_omega + 64 * static_cast<int64_t>(c_.tile) - 1) / (64 * static_cast<int64_t>(c_.tile));
   const int64_t tile = c_.tile * group, gran = group > 1 ? tile : c_.gran;
@@ -151,7 +153,7 @@ __device__ void node_plan(const Params &P, NodeCost c_) {
     if (c_.pow2) runlen = exp2f(floorf(log2f(runlen)));
     const float runs = block_sum(cnt > 0.f ? 1.f / runlen : 0.f) / windows;
     const float part = c_.part(end - t0, runs) + static_cast<float>(group - 1) * (c_.fixed + c_.per_run * runs);
-    const float total = c_.spread(done + part, fmaxf(top, part)) + c_.direct * static_cast<float>(P.n_omega - end) +
+    const float total = c_.spread(done + part, fmaxf(top, part)) + c_.direct * items(P.n_omega - end) +
                         (end < P.n_omega ? c_.second : 0.f);
     if (total < best) {
       best = total;
