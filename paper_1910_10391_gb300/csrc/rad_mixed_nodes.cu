@@ -10,8 +10,10 @@
 //   F(w_j) = sum_{c < 8} K((w_j - w_m)/h) sum_k [psi(h a_k) f_k] e^{i w_m a_k},  m = m_j + c
 // with node spacing h, twofold oversampling |h a_k| <= pi/2, K the Kaiser-Bessel window of 8 nodes
 // and psi the reciprocal of its Fourier transform. The truncation error is below 2.6e-7 of |f_k|
-// per sample, and the phases that sin/cos see stay below about 90 rad from the run's centre, where
-// the direct form has up to some hundred rad from its tile's centre.
+// per sample. The phases that sin/cos see are those of the nodes about the band's centre, at most 50 rad, and of the
+// centre about the run's, at most (w_c / h) pi / 2: 50 rad in a tile that starts near zero, up to 6400 in a band
+// narrow against its energies (h is w_hi / 4096 at least), but never more than the window's range of phases, which the direct
+// form sees. Errors in both: tests/test_run_precision_gpu.py.
 //
 // Work split: a block of 4 warps takes one direction and 128 R photon energies. Per window of 256
 // samples (the pre-pass's time tiles) each warp prepares 64 samples, cuts them into the longest

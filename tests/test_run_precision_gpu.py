@@ -35,7 +35,8 @@ def case(kind, mode):
         grid = I.make_grid(I.omega_linear(96, 1.2 * I.undulator_first_harmonic_eV(1000.0, 0.5e-10, 10e-6)), 4, 4, 2e-3)
     else:
         tr = I.channeling(2, 10e9, +1, 3000, 5e-9, 3)
-        hw = {"positrons": I.omega_log(96, 1e6, 1e9), "top": np.linspace(0.95e8, 1e8, 96)}[kind]
+        hw = {"positrons": I.omega_log(96, 1e6, 1e9), "top": np.linspace(0.95e8, 1e8, 96),
+              "narrow": np.linspace(4e9, 4.004e9, 96)}[kind]
         grid = I.Grid(hw, *directions(16))
     return tr, grid, exact_cube(tr, grid, mode)
 
@@ -110,3 +111,10 @@ def test_long_trajectory_in_one_piece(form):
     p.close()
     print(err)
     assert all(r <= max(1.1 * d, 4.4e-16) for r, d in zip(err[inp.n_omega], err[0])), err
+
+
+@pytest.mark.parametrize("mode", [rad.RAD_CLASSICAL, rad.RAD_SPIN_HALF])
+def test_nodes_of_a_narrow_band(mode):
+    """A band far above its width: the node form's phases about a run's centre reach (centre / spacing) pi / 2, up to the
+    whole range that the direct form sees from its window's reference, and its error stays below that form's."""
+    test_no_further_from_the_exact_sum_than_directly(rad.RAD_MIXED, "narrow", mode)
