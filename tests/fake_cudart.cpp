@@ -16,6 +16,7 @@ std::map<std::string, int> g_launches;
 int g_occupancy = 2;
 float g_elapsed = 1.f;
 dim3 g_grid, g_block;
+void *g_set_args = nullptr;  // where the last training step's arguments went
 }  // namespace
 
 extern "C" {
@@ -33,6 +34,7 @@ int fake_launches(const char *part, int reset) {
   if (reset) g_launches.clear();
   return n;
 }
+void *fake_set_args() { return g_set_args; }
 void fake_elapsed(float ms) { g_elapsed = ms; }
 
 cudaError_t cudaMalloc(void **p, size_t n) {
@@ -96,16 +98,28 @@ cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
-// not used by these tests: streams, capture, graphs, symbols
-cudaError_t cudaStreamCreateWithFlags(cudaStream_t *, unsigned) { return cudaErrorNotSupported; }
-cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaErrorNotSupported; }
-cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaErrorNotSupported; }
-cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *) { return cudaErrorNotSupported; }
-cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *) { return cudaErrorNotSupported; }
-cudaError_t cudaGraphInstantiate(cudaGraphExec_t *, cudaGraph_t, unsigned long long) { return cudaErrorNotSupported; }
-cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaErrorNotSupported; }
-cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaErrorNotSupported; }
-cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaErrorNotSupported; }
+// captures and graphs end well and do nothing
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) {
+  *s = reinterpret_cast<cudaStream_t>(1);
+  return cudaSuccess;
+}
+cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaSuccess; }
+cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *g) {
+  *g = reinterpret_cast<cudaGraph_t>(1);
+  return cudaSuccess;
+}
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *s) {
+  *s = cudaStreamCaptureStatusNone;
+  return cudaSuccess;
+}
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t *x, cudaGraph_t, unsigned long long) {
+  *x = reinterpret_cast<cudaGraphExec_t>(1);
+  return cudaSuccess;
+}
+cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
+cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
 cudaError_t cudaGetSymbolAddress(void **, const void *) { return cudaErrorNotSupported; }
 
 // what nvcc's generated host code calls
@@ -135,9 +149,11 @@ cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *host) {
   *k = reinterpret_cast<cudaKernel_t>(const_cast<void *>(host));
   return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3 b, void **, size_t, cudaStream_t) {
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3 b, void **args, size_t, cudaStream_t) {
   if (!g.x || !g.y || !g.z || !b.x || !b.y || !b.z || g.y > 65535 || g.z > 65535) return cudaErrorInvalidConfiguration;
-  ++g_launches[g_names[reinterpret_cast<const void *>(k)]];
+  const std::string &name = g_names[reinterpret_cast<const void *>(k)];
+  ++g_launches[name];
+  if (name.find("k_set_args") != std::string::npos) std::memcpy(&g_set_args, args[1], sizeof g_set_args);
   return cudaSuccess;
 }
 cudaError_t cudaLaunchKernel(const void *f, dim3 g, dim3 b, void **a, size_t s, cudaStream_t st) {

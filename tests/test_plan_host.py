@@ -123,3 +123,25 @@ assert before["cut"] == "auto"
 assert f.lib.rad_plan_autotune(h, *f.args(), 0, None) == 0
 assert f.describe(h) == before, (before, f.describe(h))
 """)
+
+
+def test_training_graphs_have_their_own_arguments(fake):
+    """Steps of two batch sizes may be in flight on two streams: the graph of one must not find the other's pointers."""
+    fake_gpu.run(fake, """
+import ctypes
+P, i64, c, fl = ctypes.c_void_p, ctypes.c_int64, ctypes.c_int, ctypes.c_float
+f.lib.rad_mlp_create.argtypes = [c, c, c, c, i64, ctypes.c_uint64, ctypes.POINTER(P)]
+f.lib.rad_mlp_train_step.argtypes = [P, P, P, P, i64, fl, fl, P, P]
+f.lib.fake_set_args.restype = P
+h, x = P(), P(1 << 20)
+assert f.lib.rad_mlp_create(3, 66, 2, 34, 600, 1, ctypes.byref(h)) == 0
+where = {}
+for batch in [600] * 3 + [33] * 3 + [600, 33, 1, 1, 1, 2, 2, 2, 5, 5, 5, 600, 600, 600]:
+    f.lib.fake_launches(b"", 1)
+    assert f.lib.rad_mlp_train_step(h, x, x, None, batch, 1e-3, 0.0, None, None) == 0
+    if f.lib.fake_launches(b"k_set_args", 0):
+        where.setdefault(batch, set()).add(f.lib.fake_set_args())
+assert set(where) == {600, 33, 1, 2, 5}, where
+seen = [a for s in where.values() for a in s]
+assert len(seen) == len(set(seen)) == 6, where  # 600 was replaced and built again, with arguments of its own
+""")
