@@ -41,7 +41,7 @@ SHAPES = {0: (2, 8, 256), 2: (2, 8, 256)}
 SPLIT = {0: 6, 2: 0}
 # per model: FP64 instructions per term of k_fp64 and k_df, and warp instructions per 32 terms of
 # k_df, counted by ncu (smsp__inst_executed_pipe_fp64.sum x 32 / terms, smsp__inst_executed.sum)
-# on the launch these legs time: one particle of this workload x 512 hw x 64x64 directions, the
+# with every energy summed directly: one particle of this workload x 512 hw x 64x64 directions in the
 # default shapes (k_fp64 R=2 NW=8 T=64, k_df R=2 NW=4 T=64)
 FP64_OPS_PER_TERM = {0: 18.53, 2: 20.58}
 DF_INST_PER_32_TERMS = {0: 134.5, 2: 159.3}

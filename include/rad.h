@@ -114,8 +114,12 @@ extern "C" {
  * n_omega or n_angles exceeds 2^31, or when the call would split into more than about 2^31
  * work items (RAD_FP64_DF takes one direction per item: at most about 2^31 directions per 256
  * photon energies).
- * Scratch memory is allocated by the library on first use of a shape and reused
- * (see rad_release). Thread-safe; concurrent calls on different streams are allowed.
+ * Scratch memory is allocated by the library on first use of a shape and reused: one plan per
+ * shape and stream, each kept until rad_release. A plan holds a cube, the partial sums (at most
+ * 4 GiB), in RAD_MIXED 48 bytes per sample and, where RAD_FP64 or RAD_FP64_DF may sum the lowest
+ * energies through Chebyshev moments (see rad_plan_set_cut), up to 410 MB of amplitudes (1.35 MB
+ * per resident block at 512 energies) and up to 512 MB more partial sums; without room for these
+ * the plan is the term-by-term kernel's. Thread-safe; concurrent calls on different streams are allowed.
  */
 int rad_spectrum(const double *samples, int64_t n_samples_total, const int64_t *offsets,
                  int64_t n_particles, const double *gamma, const double *energy_eV,
@@ -247,6 +251,8 @@ int rad_plan_autotune(rad_plan plan, const double *samples, const int64_t *offse
  *               direction and each warp its own 32 R energies (NW x 32 R energies per item)
  *   T           time-tile length (FP64, FP64_DF: 64; mixed: 64, 128 or 256)
  *   chunk_mult  >= 1, multiplies the default number of work items (finer split)
+ * The shape is that of the term-by-term kernel; any but a new plan's own (R, NW, T) also sends
+ * every energy through it (see rad_plan_set_cut).
  * Returns RAD_EINVAL for a shape this build does not provide (the plan is unchanged).
  * May reallocate scratch (waits for the device); not allowed during stream capture.
  */
@@ -266,7 +272,8 @@ int rad_plan_set_prepass(rad_plan plan, int enable);
  * terms whose index is every - 1 mod every in each group of 8 samples x R energies (R = 2: 1/4 or
  * 1/8 of them) on the FMA pipe (Cody-Waite reduction to |r| <= pi/4, Taylor polynomials; same
  * error bound as the SFU's on the in-tile phases) instead of the SFU, so that both pipes share
- * the work; 0 uses the SFU for every term. A new plan starts with 6 for the classical and spin-0
+ * the work; 0 uses the SFU for every term. It concerns the energies that this kernel sums: all of
+ * them, or those above the cut (see rad_plan_set_cut). A new plan starts with 6 for the classical and spin-0
  * models and 0 for spin-1/2. RAD_EINVAL for other values, FP64 plans or the inline-preparation
  * kernel (plan unchanged). The autotuner also tries these.
  */
@@ -312,10 +319,10 @@ int rad_plan_describe(rad_plan plan, char *buf, int len);
 
 /*
  * rad_plan_set_timing -- enable != 0 makes every later rad_plan_execute of this plan
- * record CUDA events on its stream just before and after the main integral kernel (after
- * the mixed kernel's per-sample pre-pass, which is not included);
- * rad_plan_last_kernel_ms waits for the last recorded pair and returns the main
- * kernel's duration in milliseconds in *ms. Do not enable timing on a plan that is
+ * record CUDA events on its stream just before and after the integral kernels (term by term
+ * and, with a cut, the other; after the mixed kernel's per-sample pre-pass, which is not included);
+ * rad_plan_last_kernel_ms waits for the last recorded pair and returns their
+ * duration in milliseconds in *ms. Do not enable timing on a plan that is
  * captured into a graph.
  */
 int rad_plan_set_timing(rad_plan plan, int enable);

@@ -24,14 +24,14 @@
 // (products by FMA, Ogita-Rump-Oishi Dot2 sums), because GB300 executes FP64 at 1/64 of its FP32
 // rate: a float-pair multiply-add takes about a sixth of the time of an FP64 one.
 //
-// What bounds it: the FP64 pipe (79-90 % busy) in FP64; latency at 8 warps an SM in float pairs (255
-// registers a thread hold the moments; IPC 1.7). Measured, all kernels of a call, before (direct kernel
-// alone) and with it: one undulator, 4096 samples x 128 energies x 256 directions, FP64, 4.49 -> 0.50
-// ms; 64 sections of 500 samples x 192 log energies x 324 directions, spin 1/2, FP64, 80.9 -> 39.1 ms
-// (the 64 highest energies stay direct: 25.7 ms of it); 20 undulator periods, 40960 samples x 500
-// energies x 225 directions, float pairs, 21.6 -> 5.1 ms; 6 positrons x 12000 samples x 384 log energies
-// x 576 directions, spin 1/2, float pairs, 108 -> 56 ms. Tried and slower: 28 moments for spin 1/2 (41.1
-// against 39.6 ms, and spills in float pairs), 24 for the other models (5.6 -> 7.2 ms).
+// What bounds it: the FP64 pipe (86 % busy on the sections below) in FP64; latency at 8 warps an SM in float pairs
+// (255 registers a thread hold the moments, with 40 to 76 bytes of spills; 48 % of the issue slots). Measured, all kernels
+// of a call, before (direct kernel alone) and with it: one undulator, 4096 samples x 128 energies x 256 directions, FP64, 4.49
+// -> 0.46 to 0.56 ms (from run to run); 64 sections of 500 samples x 192 log energies x 324 directions, spin 1/2, FP64, 80.9 ->
+// 41.8 ms (the 64 highest energies stay direct: 25.7 ms of it); 20 undulator periods, 40960 samples x 500 energies x 225
+// directions, float pairs, 21.6 -> 5.2 ms; 6 positrons x 12000 samples x 384 log energies x 576 directions, spin 1/2, float
+// pairs, 108 -> 57 ms. Tried and slower: 28 moments for spin 1/2 (41.1 against 39.6 ms, and spills in float pairs), 24
+// for the other models (5.6 -> 7.2 ms); 4 KB of base phases in shared memory instead of 1 (one block an SM in spin 1/2).
 #include <type_traits>
 
 #include "rad_df_reduce.cuh"

@@ -24,12 +24,13 @@
 // directly and the interpolation of one energy about as much as 5 samples, so the form pays where
 // runs are long against 5 samples and energies many against 30.
 //
-// What bounds it: shared-memory wavefronts (76 % of the peak) and issue slots. Measured, all kernels of
+// What bounds it: shared-memory wavefronts (64 % of the peak on the ensemble below, 76 % on the labels) and issue slots
+// (59 %), with 15 warps an SM to hide the latency of either. Measured, all kernels of
 // a call, before (k_mixed_pp alone) and with it: 32 positrons x 20000 samples x 512 log energies x 4096
 // directions 546 -> 158 ms; 64 electrons of 2000 to 200000 samples x 1024 energies x 576 directions,
-// spin 1/2, 482 -> 180 ms; 64 particles x 8192 samples x 256 energies x 512 directions with 15 rad per
+// spin 1/2, 437 -> 187 ms; 64 particles x 8192 samples x 256 energies x 512 directions with 15 rad per
 // sample at the top (where the upper energies stay direct) 30.7 -> 19.5 ms; one undulator of 4096
-// samples x 128 energies x 256 directions 135 -> 94 us. Tried and slower: window values in registers
+// samples x 128 energies x 256 directions 135 -> 96 us. Tried and slower: window values in registers
 // (168 of them, spills), 3 blocks an SM, node sums per sample instead of per pair of samples.
 #include "rad_mixed_common.cuh"
 

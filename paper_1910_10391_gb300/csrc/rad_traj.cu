@@ -385,7 +385,7 @@ __device__ __forceinline__ State deriv_axial(const Chan &C, const Axial &A, doub
 
 // ------------------------------------------------------------------------------------
 // Pieces of the tabulated and of the lane-group kernels: FP64 divisions and square roots cost some
-// ten dependent instructions each, and a step is one dependent chain.
+// ten dependent instructions each, and a step is one dependent chain, so that a stage shares its reciprocals.
 // ------------------------------------------------------------------------------------
 // What a stage needs of the energy: g, 1/E, 1/g^2 and the energy part of the longitudinal velocity
 // (1/g0^2 - 1/g^2 and 1 - 1/g^2)
@@ -606,13 +606,13 @@ __device__ __forceinline__ AxialStage axial_stage(const Chan &C, const EnergyPar
   return AxialStage{Fx * e.inv_E, Fy * e.inv_E, dz, C.ll ? C.ll_k * (e.g * e.g) * fma(Fx, Fx, Fy * Fy) : 0.0};
 }
 
-// The record's force is the first stage's, so a step evaluates the force four times; the divisions
-// and roots of the kinematics are the short forms above, and every lane draws the kick of one of the
+// The record's force is the first stage's, so a step evaluates the force four times; the kinematics
+// multiply by reciprocals that a stage or a step shares, and every lane draws the kick of one of the
 // next W steps. W = 32 lanes per particle as long as every warp has an SM sub-partition of its own
 // (sub_partitions): an FP64 instruction occupies the sub-partition for 64 clocks whatever its active lanes,
 // so the time of a step is the number of FP64 instructions of a warp. 512 particles x 1000 steps of the
-// <110> axis: 73.6 ms with 128-thread blocks, five force sums a step and IEEE divisions; 35.7 ms with
-// these taken out, on 16 lanes; 23.1 ms on 32. (Tried and slower: branch-free exponentials and masked
+// <110> axis: 73.6 ms with 128-thread blocks, five force sums a step and a division each; 35.7 ms with
+// these taken out, on 16 lanes; 23.3 ms on 32. (Tried and slower: branch-free exponentials and masked
 // image loops, 38.2 against 35.7 ms.)
 template <int W>
 __global__ void k_axial_group(const Chan C, const Axial A, int64_t n_particles, const int64_t *__restrict__ offsets,
