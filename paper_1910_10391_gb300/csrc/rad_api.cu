@@ -161,7 +161,8 @@ NodeCost route_cost(rad_plan p) {
 // Whether any number of energies could be worth the node or moment kernel, whatever the trajectories: with runs of the
 // largest length, whole tiles at a time and the last one up to the end. What this excludes, the choice on the device
 // (node_plan in rad_post.cu, with the same costs and margin) leaves to the direct kernel in every call.
-bool route_may_pay(const NodeCost &nc, int64_t n_omega) {
+bool route_may_pay(NodeCost nc, int64_t n_omega) {
+  if (nc.setup_if_differ) nc.setup = 0.f;  // the particle energies may be equal
   auto items = [&](int64_t n) { return static_cast<double>((n + nc.gran - 1) / nc.gran * nc.gran); };
   const double direct = 1.001 * nc.margin * nc.direct * items(n_omega);
   double total = 0.0;

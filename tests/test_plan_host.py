@@ -67,7 +67,7 @@ print(sorted(seen), least, need)
 SMALL = [(1478, 7, 80, 16, 2, 0), (1478, 7, 80, 33, 2, 2), (340, 2, 512, 16, 0, 0), (340, 2, 513, 16, 0, 2), (1031, 1, 130, 40, 2, 2),
          (1468, 4, 129, 25, 0, 1), (2999, 1, 160, 16, 2, 1), (512, 1, 96, 16, 0, 1), (4000, 2, 24, 16, 0, 0)]
 LARGE = [(4096, 1, 128, 256, 0, 0), (4096, 1, 128, 256, 0, 1), (40961, 1, 500, 225, 0, 2), (32000, 64, 192, 324, 2, 0),
-         (72000, 6, 384, 576, 2, 2), (640000, 32, 512, 4096, 0, 1), (524288, 64, 256, 512, 2, 1)]
+         (72000, 6, 384, 576, 2, 2), (640000, 32, 512, 4096, 0, 1), (524288, 64, 256, 512, 2, 1), (19200, 64, 512, 1024, 2, 1)]
 
 
 def test_calls_that_cannot_gain_are_the_direct_kernels(fake):
