@@ -292,7 +292,7 @@ int rad_plan_set_sincos_split(rad_plan plan, int every);
  * particles, and other launch shapes (the plan is unchanged). May reallocate scratch, as
  * rad_plan_set_shape. rad_plan_describe shows it as cut=auto, cut=0 or the number.
  * rad_plan_last_cut -- the number of the last execute (waits for the device), RAD_EINVAL before
- * the first one.
+ * the first one since the plan was made or changed.
  */
 int rad_plan_set_cut(rad_plan plan, int64_t n_lowest);
 int rad_plan_last_cut(rad_plan plan, int64_t *n_lowest);

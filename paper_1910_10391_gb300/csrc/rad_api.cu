@@ -125,9 +125,13 @@ constexpr int64_t kChebMinFp64 = 24, kChebMinDf = 64;
 // Partials that a finer split for the moment kernel may take (doubles).
 constexpr int64_t kChebPartials = int64_t(1) << 26;
 
+// What a second kernel's start and end take beside the first one's (15 us; calls of 12000 samples and 20 to 36 directions came
+// out best with it, 5 us sent some to their loss, 25 us kept others from a gain).
 constexpr double kSecondKernelClocks = 30e3;
 
-// Costs of the plan's node or moment kernel, for the choice of the cut.
+// Costs of the plan's node or moment kernel, for the choice of the cut. Blocks that fill the GPU: two per SM of the moment
+// kernel in float pairs and four of the node kernel hide each other's latency; in FP64 a block alone on its SM reaches two
+// thirds of the rate of two.
 NodeCost route_cost(rad_plan p) {
   NodeCost nc;
   int64_t items, slots;  // of one energy tile; blocks that fill the GPU
@@ -289,6 +293,7 @@ int configure(rad_plan p, const Choice &c, bool moments = true) {
   sh.grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(p->n_items, resident)));
   p->shape = sh;
   p->choice = c;
+  p->ran = false;
   p->nodes = p->precision == RAD_MIXED ? moments && c.pp && def_shape && node_path_allowed(sh, p->n_omega, p->n_angles, p->n_chunks)
                                        : cheb && ctiles <= (INT32_MAX - 65536) / p->n_chunks;
   if (p->nodes && p->set_cut < 0 && !route_may_pay(route_cost(p), p->n_omega)) {
@@ -316,10 +321,6 @@ int configure(rad_plan p, const Choice &c, bool moments = true) {
       }
       p->cheb_cap = bytes;
     }
-  } else if (p->cheb_scratch) {  // the partials may need its room
-    cudaFree(p->cheb_scratch);
-    p->cheb_scratch = nullptr;
-    p->cheb_cap = 0;
   }
   const size_t need = static_cast<size_t>(std::max<int64_t>(per_chunk * p->n_chunks, 1));
   if (need > p->part_cap) {
@@ -327,8 +328,11 @@ int configure(rad_plan p, const Choice &c, bool moments = true) {
     p->part = nullptr;
     p->part_cap = 0;
     cudaError_t e = cudaMalloc(&p->part, need * sizeof(double));
-    if (e != cudaSuccess && cheb) {  // no room for the finer split: the direct kernel alone
+    if (e != cudaSuccess && (cheb || p->cheb_scratch)) {  // no room beside the moment kernel: the direct kernel alone
       (void)cudaGetLastError();
+      cudaFree(p->cheb_scratch);
+      p->cheb_scratch = nullptr;
+      p->cheb_cap = 0;
       return configure(p, c, false);
     }
     if (e != cudaSuccess) return cuda_fail(e);
