@@ -25,7 +25,7 @@ __device__ void node_plan(const Params &P, NodeCost c_) {
   const int tid = threadIdx.x;
   bool bad = false;
   for (int64_t i = tid; i + 1 < P.n_omega; i += 256) bad |= !(P.hw[i] <= P.hw[i + 1]);
-  // the calls' longest trajectory against the mean: with few work items it is the last to end
+  // the call's longest trajectory against the mean: with few work items it is the last to end
   int64_t longest = 0;
   for (int64_t p = tid; p < P.n_particles; p += 256) {
     const int64_t n = P.offsets[p + 1] - P.offsets[p];
@@ -36,7 +36,7 @@ __device__ void node_plan(const Params &P, NodeCost c_) {
   // steps in phase length of window `at` (of 16) of particle p; false where the records are not usable
   auto window = [&](int64_t p, int at, const double *&w0, int64_t &span) {
     const int64_t ka = P.offsets[p], kb = P.offsets[p + 1], n = kb - ka;
-    if (ka < 0 || n < 2 || kb > P.n_samples_total) return false;
+    if (ka < 0 || kb < 0 || n < 2 || kb > P.n_samples_total) return false;  // kb < 0: n may have wrapped
     span = n < 256 ? n : 256;
     w0 = P.samples + (ka + (n - span) * at / 15) * kRec;
     return true;
