@@ -757,9 +757,11 @@ inline bool tab_fits(const Planar &P, const Chan &C) {
   const double h = C.d_p / kTabI;
   double most = 0.0, least = INFINITY, least_el = INFINITY;
   for (int i = 0; i < P.nt; ++i) {
-    most = fmax(most, P.ck[i]);
-    least = fmin(least, P.ck[i]);
-    if (P.el) {
+    if (P.fk[i] != 0.0) {
+      most = fmax(most, P.ck[i]);
+      least = fmin(least, P.ck[i]);
+    }
+    if (P.el && P.ek[i] != 0.0) {
       most = fmax(most, P.eck[i]);
       least_el = fmin(least_el, P.eck[i]);
     }

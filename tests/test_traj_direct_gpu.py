@@ -58,3 +58,16 @@ def test_no_wide_term(n, kd2):
     ch = rad.RadChannel(0.0, D_P, I.EPS_S_EV, I.SI_X0, rho, I.ME_EV, +1, 0)
     got, _, off = run_gpu(ch, lib, x0, np.zeros(n), E, np.full(n, L), dt, 1)
     check(got, off, range(24), x0, np.zeros(n), E, L, dt, 1, +1, 0, orc, rho)
+
+
+def test_wide_term_without_weight():
+    """A padded fit: the wide Gaussian has no amplitude, the narrow one's tail is the force between the planes."""
+    E, dt, L, n = 20e9, 5e-9, 40, 24
+    rho = D_P / math.sqrt(600.0)
+    a, b = (3e-10, 0.0), (0.0, 4e-20)
+    lib = rad.RadPlanarPotential.make(a, b, I.SI_N, n_neighbours=2)
+    orc = T.PlanarPotential(a, b, I.SI_N, K=2)
+    x0 = np.linspace(0.05, 0.48, n) * D_P
+    ch = rad.RadChannel(0.0, D_P, I.EPS_S_EV, I.SI_X0, rho, I.ME_EV, +1, 0)
+    got, _, off = run_gpu(ch, lib, x0, np.zeros(n), E, np.full(n, L), dt, 1)
+    check(got, off, range(n), x0, np.zeros(n), E, L, dt, 1, +1, 0, orc, rho)
