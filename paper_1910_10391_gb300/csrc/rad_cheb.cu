@@ -25,7 +25,7 @@
 // rate: a float-pair multiply-add takes about a sixth of the time of an FP64 one.
 //
 // What bounds it: the FP64 pipe (86 % busy on the sections below) in FP64; latency at 8 warps an SM in float pairs
-// (255 registers a thread hold the moments, with 40 to 76 bytes of spills; 48 % of the issue slots). Measured, all kernels
+// (255 registers a thread hold the moments, with 60 to 76 bytes of spill stores; 48 % of the issue slots). Measured, all kernels
 // of a call, before (direct kernel alone) and with it: one undulator, 4096 samples x 128 energies x 256 directions, FP64, 4.49
 // -> 0.46 to 0.56 ms (from run to run); 64 sections of 500 samples x 192 log energies x 324 directions, spin 1/2, FP64, 80.9 ->
 // 41.8 ms (the 64 highest energies stay direct: 25.7 ms of it); 20 undulator periods, 40960 samples x 500 energies x 225
